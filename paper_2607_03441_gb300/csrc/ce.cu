@@ -25,17 +25,18 @@
 namespace attt {
 
 constexpr int kCeBN = 256;
-constexpr int kCeMaxTiles = 256;  // vocab tiles per chunk at most
-constexpr int kChunkWarps = 8;  // ce_chunk_kernel: 8 warps, 32 rows (one per lane) per block
+constexpr int kCeMinBN = 64;      // the narrowest tile of the logits contraction
+constexpr int kCeMaxTiles = 1024;  // chunk width at most, in kCeBN columns
+constexpr int kChunkWarps = 16;  // ce_chunk_kernel: 16 warps, 32 rows (one per lane) per block
 constexpr int kChunkRows = 32;
-// fp32 partials of 128 x kCeBN (128 KB each) for the tail split of the dh
-// contraction: enough for every CTA of a 160-SM part to hold one piece.
-constexpr int kCeSplitRegions = 160;
+// fp32 partials of 128 x kCeBN (128 KB each) for the K pieces of the dh
+// contraction (40 MB): two pieces for every SM of a 160-SM part.
+constexpr int kCeSplitRegions = 320;
 // Bound of the chunk's bf16 block E [L, Vc] in bytes.
 constexpr int64_t kCeEBytes = 1024ll << 20;
 
 struct CeLayout {
-    int64_t nvt, Vc, nblk;
+    int64_t Vc, nblk;
     float2 *part;
     float *ztgt, *block_sums;
     float *aref, *mref, *lm, *ls, *alpha, *beta, *gamma;
@@ -50,7 +51,9 @@ struct CeLayout {
 // Upper bound of the vocab chunk: the chunk's bf16 block E (L x Vc) is kept
 // near kCeEBytes (1 GB), so the workspace stays bounded whatever V is.  Each chunk costs
 // about 20 us of launch, ramp and tail on top of its FLOPs, and E is streamed
-// once from L2 or HBM either way, so wider chunks are faster up to this bound.
+// once from L2 or HBM either way, so wider chunks are faster up to this bound
+// (d 3,584, V 152,064, one chunk against three: L 93 354 against 415 us, L 403
+// 660 against 796, L 2,048 2,350 against 2,390).
 static int64_t ce_chunk_max(int64_t L, int64_t V) {
     int64_t vc = kCeEBytes / (2 * L);
     vc = (vc / kCeBN) * kCeBN;
@@ -61,53 +64,31 @@ static int64_t ce_chunk_max(int64_t L, int64_t V) {
     return vc;
 }
 
-// Tile plan for `sms` SMs.  Above 128 rows both contractions run on CTA pairs
-// (cta_group::2: 256 x 256 accumulator tiles), else on single CTAs (128 x 256).
-// The chunk width Vc (<= the workspace bound) minimises an estimate of the
-// time that counts whole waves of tiles (a partial wave costs a full one)
-// plus a per-launch cost.
+// Chunk width and the tiles of both contractions for `sms` SMs.
 struct CePlan {
     int64_t Vc;
-    bool pair;
+    TilePlan logits, dh;
 };
 
-static CePlan ce_plan(int64_t L, int64_t d, int64_t V, int sms) {
-    const double rate = 1.0e13;    // bf16 FLOP/s of one SM, order of magnitude
-    const double launch = 7.0e-6;  // seconds per launch, ramp-up and tail included
-    const bool pair = L > 128;
-    const int64_t rows = pair ? 256 : 128;       // accumulator rows per tile
-    const int64_t units = pair ? sms / 2 : sms;  // tiles in flight
-    const double tile_rate = rate * (pair ? 2.0 : 1.0);
-    const int64_t tm = cdiv(L, rows);
-    const double w2 = (double)cdiv(tm * cdiv(d, kCeBN), units);
-    CePlan best{ce_chunk_max(L, V), pair};
-    double best_t = 1e30;
-    const int64_t vmax = ce_chunk_max(L, V);
-    for (int64_t vc = 4 * kCeBN; vc <= vmax; vc += kCeBN) {
-        double t = 0.0;
-        for (int64_t v0 = 0; v0 < V; v0 += vc) {
-            const int64_t nc = (V - v0 < vc) ? V - v0 : vc;
-            const double w1 = (double)cdiv(tm * cdiv(nc, kCeBN), units);
-            t += (w1 * d + w2 * round_up(nc, 64)) * 2.0 * rows * kCeBN / tile_rate + 3 * launch;
-        }
-        if (t < best_t) { best_t = t; best = CePlan{vc, pair}; }
-        if (vc == vmax) break;
-    }
-    return best;
+static CePlan ce_plan(int64_t L, int64_t d, int64_t V, int regions, int sms) {
+    CePlan p{};
+    const int64_t nchunks = cdiv(V, ce_chunk_max(L, V));
+    p.Vc = round_up(cdiv(V, nchunks), kCeBN);  // equal chunks
+    p.logits = plan_tiles(L, p.Vc, cdiv(d, 64), sms, 0, false, false);
+    p.dh = plan_tiles(L, d, cdiv(p.Vc, 64), sms, regions, true, true);
+    return p;
 }
 
 static CeLayout ce_layout(void *ws, int64_t L, int64_t d, int64_t V) {
     CeLayout c{};
-    // tail split of the dh contraction: at most 4 pieces per tile and 2 CTAs
-    // per tile, so 8 regions per tile of the contraction bound the need
-    const int64_t rows = L > 128 ? 256 : 128;
-    const int64_t t2 = cdiv(L, rows) * cdiv(d, kCeBN);
-    c.split_regions = (int)(8 * t2 < kCeSplitRegions ? 8 * t2 : kCeSplitRegions);
-    c.nvt = cdiv(V, kCeBN);
+    // K pieces of the dh contraction: at most kMaxPieces per tile, of at most
+    // two 128-row regions per 256 rows
+    const int64_t t2 = 2 * kMaxPieces * cdiv(L, 256) * cdiv(d, kCeBN);
+    c.split_regions = (int)(t2 < kCeSplitRegions ? t2 : kCeSplitRegions);
     c.Vc = ce_chunk_max(L, V);
     c.nblk = cdiv(L, kChunkRows);
     Carve cv{static_cast<char *>(ws), 0};
-    c.part = cv.take<float2>((size_t)(c.nvt * L));
+    c.part = cv.take<float2>((size_t)(cdiv(c.Vc, kCeMinBN) * L));
     c.ztgt = cv.take<float>((size_t)L);
     c.block_sums = cv.take<float>((size_t)c.nblk);
     c.aref = cv.take<float>((size_t)L);
@@ -140,8 +121,11 @@ __device__ __forceinline__ void lse_merge(float &m, float &s, float m2, float s2
 __global__ void __launch_bounds__(256) ce_ref_kernel(const __nv_bfloat16 *__restrict__ h,
                                                      const __nv_bfloat16 *__restrict__ W,
                                                      const int32_t *__restrict__ tgt, int L, int64_t d, int V,
-                                                     float *__restrict__ mref) {
+                                                     float *__restrict__ mref, unsigned int *__restrict__ tick,
+                                                     int ntick) {
     griddep_launch_dependents();  // the first logits contraction may start its main loop
+    if (blockIdx.x == 0)  // the call's arrival counters start at zero
+        for (int i = threadIdx.x; i < ntick; i += blockDim.x) tick[i] = 0u;
     const int j = blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (j >= L) return;
@@ -170,8 +154,8 @@ __global__ void __launch_bounds__(256) ce_ref_kernel(const __nv_bfloat16 *__rest
 }
 
 struct CeChunkArgs {
-    const float2 *part;  // [vocab tiles, L] (max, sum) of every tile (log2 units)
-    int tile0, ntiles, L, V;
+    const float2 *part;  // [vocab tiles of the chunk, L] (max, sum) of every tile (log2 units)
+    int ntiles, tile_w, L, V;  // tile_w: columns per tile
     __nv_bfloat16 *G;
     int64_t G_ld;
     float *aref, *mref, *lm, *ls, *alpha, *beta, *gamma;
@@ -191,9 +175,10 @@ struct CeChunkArgs {
 };
 
 // Bookkeeping of one chunk, 32 rows per block (lane = row), log2 units:
-//   warp k reads the chunk's tiles t = k (mod 8) with coalesced loads of
-//   part[t, rows]; per row the chunk max M_c and the chunk's (max, sum) pair,
-//   merged into the running pair (lm, ls);
+//   warp k reads the chunk's tiles t = k (mod 16) with coalesced loads of
+//   part[t, rows], four in flight (one chunk may hold 600 tiles and few rows:
+//   the loads' latency bounds the kernel); per row the chunk max M_c and the
+//   chunk's (max, sum) pair, merged into the running pair (lm, ls);
 //   R = mref, the reference GEMM1 wrote this chunk's E against.  A tile whose
 //   max exceeded R by more than kCeRefJump used its own max, and then
 //   (M_c - R > kCeRefJump) the row is rewritten against M_c tile by tile
@@ -201,11 +186,11 @@ struct CeChunkArgs {
 //   acc = alpha * acc + beta * (E W_c) with A_new = max(A_old, Rp),
 //   alpha = exp2(A_old - A_new), beta = exp2(Rp - A_new);  mref <- max(R, M_c).
 // Last chunk: lse = ln 2 (lm + log2 ls); the weighted NLL of the block's rows
-// goes to block_sums and the last block (ticket) adds them in block order;
+// goes to block_sums and the last block (ticket) adds them in a fixed order;
 // alpha and beta take the factor (w/L) exp2(A_new - lse log2 e) and gamma =
 // w/L, so the last GEMM2 writes dh itself.
 __global__ void __launch_bounds__(kChunkWarps * 32) ce_chunk_kernel(const CeChunkArgs a) {
-    __shared__ float s_mc[kChunkWarps][kChunkRows], s_m[kChunkWarps][kChunkRows], s_s[kChunkWarps][kChunkRows];
+    __shared__ float s_m[kChunkWarps][kChunkRows], s_s[kChunkWarps][kChunkRows];
     __shared__ float s_r[kChunkRows], s_mcf[kChunkRows];
     __shared__ int s_rw[kChunkRows];
     __shared__ bool s_last;
@@ -215,23 +200,28 @@ __global__ void __launch_bounds__(kChunkWarps * 32) ce_chunk_kernel(const CeChun
     const int j0 = blockIdx.x * kChunkRows;
     const int j = j0 + lane;
     const int L = a.L;
-    float mc = -INFINITY, m = -INFINITY, s = 0.f;
+    float m = -INFINITY, s = 0.f;
     if (j < L) {
-        for (int t = warp; t < a.ntiles; t += kChunkWarps) {
-            const float2 p = __ldcg(a.part + (int64_t)(a.tile0 + t) * L + j);
-            mc = fmaxf(mc, p.x);
-            lse_merge(m, s, p.x, p.y);
+        for (int t = warp; t < a.ntiles; t += 4 * kChunkWarps) {
+            float2 p[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                p[k] = t + k * kChunkWarps < a.ntiles ? __ldcg(a.part + (int64_t)(t + k * kChunkWarps) * L + j)
+                                                      : make_float2(-INFINITY, 0.f);
+            const float mx = fmaxf(m, fmaxf(fmaxf(p[0].x, p[1].x), fmaxf(p[2].x, p[3].x)));
+            if (mx == -INFINITY) continue;
+            s *= exp2f(m - mx);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) s += p[k].y * exp2f(p[k].x - mx);
+            m = mx;
         }
     }
-    s_mc[warp][lane] = mc;
     s_m[warp][lane] = m;
     s_s[warp][lane] = s;
     __syncthreads();
     if (warp == 0) {
-        for (int k = 1; k < kChunkWarps; ++k) {
-            mc = fmaxf(mc, s_mc[k][lane]);
-            lse_merge(m, s, s_m[k][lane], s_s[k][lane]);
-        }
+        for (int k = 1; k < kChunkWarps; ++k) lse_merge(m, s, s_m[k][lane], s_s[k][lane]);
+        const float mc = m;  // the chunk's max
         int rw = 0;
         float r = 0.f, contrib = 0.f;
         if (j < L) {
@@ -290,16 +280,16 @@ __global__ void __launch_bounds__(kChunkWarps * 32) ce_chunk_kernel(const CeChun
     }
     __syncthreads();
     // rows whose tiles used their own max: E against M_c, tile by tile
-    const int per_tile = kCeBN / 8;  // uint4 (8 x bf16) per tile row
+    const int per_tile = a.tile_w / 8;  // uint4 (8 x bf16) per tile row
     for (int i = warp; i < kChunkRows; i += kChunkWarps) {
         if (!s_rw[i]) continue;
         const int jr = j0 + i;
         const float r = s_r[i], mcr = s_mcf[i];
         uint4 *row = reinterpret_cast<uint4 *>(a.G + (int64_t)jr * a.G_ld);
         for (int t = 0; t < a.ntiles; ++t) {
-            const float mt = __ldcg(&a.part[(int64_t)(a.tile0 + t) * L + jr].x);
+            const float mt = __ldcg(&a.part[(int64_t)t * L + jr].x);
             const float sc = (mt - r > kCeRefJump) ? exp2f(mt - mcr) : exp2f(r - mcr);
-            for (int q = lane; q < per_tile; q += 32) {
+            for (int q = lane; q < per_tile && t * per_tile + q < a.G_ld / 8; q += 32) {
                 uint4 u = row[t * per_tile + q];
                 uint32_t *wd = reinterpret_cast<uint32_t *>(&u);
 #pragma unroll
@@ -313,12 +303,15 @@ __global__ void __launch_bounds__(kChunkWarps * 32) ce_chunk_kernel(const CeChun
             }
         }
     }
-    if (a.last && s_last && threadIdx.x == 0) {
+    if (a.last && s_last && warp == 0) {  // a fixed order: lane sums of blocks lane (mod 32), then a tree
         __threadfence();
         float total = 0.f;
-        for (unsigned i = 0; i < gridDim.x; ++i) total += __ldcg(a.block_sums + i);
-        *a.loss = total * a.inv_L;
-        *a.ticket = 0u;
+        for (unsigned i = lane; i < gridDim.x; i += 32) total += __ldcg(a.block_sums + i);
+        for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
+        if (lane == 0) {
+            *a.loss = total * a.inv_L;
+            *a.ticket = 0u;
+        }
     }
 }
 
@@ -344,7 +337,8 @@ size_t ce_workspace_bound(int64_t Lmax, int64_t d, int64_t V) {
     if (Lmax < 1) return 0;
     size_t best = attt_ce_workspace_bytes(Lmax, d, V);
     const int64_t budget = kCeEBytes / 2;
-    for (int64_t vc = kCeBN; vc <= kCeMaxTiles * kCeBN; vc += kCeBN) {
+    const int64_t vmax = round_up(V, kCeBN) < kCeMaxTiles * kCeBN ? round_up(V, kCeBN) : kCeMaxTiles * kCeBN;
+    for (int64_t vc = kCeBN; vc <= vmax; vc += kCeBN) {
         const int64_t L = budget / vc;  // the last L whose unclamped chunk is at least vc
         for (int64_t c = L - 1; c <= L + 1; ++c)
             if (c >= 1 && c <= Lmax) {
@@ -391,37 +385,34 @@ attt_status ce_fwd_bwd_run(const attt_bf16 *d_h, const attt_bf16 *d_W, const int
     if (!status) return ATTT_ERR_CUDA;
 
     CeLayout c = ce_layout(d_ws, L, d, V);
-    if (cudaMemsetAsync(c.ticket, 0, sizeof(unsigned int) * (4 + (size_t)c.split_regions), stream) != cudaSuccess)
-        return ATTT_ERR_CUDA;
-
     ce_ref_kernel<<<(unsigned)cdiv(L, 8), 256, 0, stream>>>(reinterpret_cast<const __nv_bfloat16 *>(d_h),
                                                             reinterpret_cast<const __nv_bfloat16 *>(d_W), d_tgt,
-                                                            (int)L, d, (int)V, c.mref);
+                                                            (int)L, d, (int)V, c.mref, c.ticket, 4 + c.split_regions);
     count_launch();
     if (cudaGetLastError() != cudaSuccess) return ATTT_ERR_CUDA;
 
-    const CePlan plan = ce_plan(L, d, V, num_sms(dev));
+    const CePlan plan = ce_plan(L, d, V, c.split_regions, num_sms(dev));
     for (int64_t v0 = 0, ci = 0; v0 < V; v0 += plan.Vc, ++ci) {
         const int64_t Nc = (V - v0 < plan.Vc) ? V - v0 : plan.Vc;
-        const int ntiles = (int)cdiv(Nc, kCeBN);
+        const int ntiles = (int)cdiv(Nc, plan.logits.BN);
         const bool last = v0 + Nc >= V;
         {   // GEMM1: logits of the chunk -> per-tile stats and E = exp(z - R)
             GemmProblem p{};
             p.a = d_h; p.a_rows_ld = d; p.a_rows = L; p.a_k = d;
             p.b = d_W; p.b_rows_ld = d; p.b_rows = V; p.b_k = d;
-            p.M = (int)L; p.N = (int)Nc; p.K = (int)d; p.BN = kCeBN; p.pair = plan.pair;
+            p.M = (int)L; p.N = (int)Nc; p.K = (int)d; p.BN = plan.logits.BN; p.pair = plan.logits.pair;
             p.b_n_off = (int)v0;
             p.pdl = true;
             p.operands_ready = true;  // h and W are inputs of the call
             EpiParams ep{};
-            ep.tgt = d_tgt; ep.part = c.part; ep.tile0 = (int)(v0 / kCeBN); ep.ztgt = c.ztgt; ep.v0 = (int)v0;
+            ep.tgt = d_tgt; ep.part = c.part; ep.tile0 = 0; ep.ztgt = c.ztgt; ep.v0 = (int)v0;
             ep.G = c.G; ep.G_ld = c.Vc;
             ep.eref = c.mref;
             st = launch_gemm<EPI_CE_EXP, false, false>(p, ep, dev, stream);
             if (st != ATTT_OK) return st;
         }
         CeChunkArgs ca{};
-        ca.part = c.part; ca.tile0 = (int)(v0 / kCeBN); ca.ntiles = ntiles; ca.L = (int)L; ca.V = (int)V;
+        ca.part = c.part; ca.ntiles = ntiles; ca.tile_w = plan.logits.BN; ca.L = (int)L; ca.V = (int)V;
         ca.G = c.G; ca.G_ld = c.Vc;
         ca.aref = c.aref; ca.mref = c.mref; ca.lm = c.lm; ca.ls = c.ls;
         ca.alpha = c.alpha; ca.beta = c.beta; ca.gamma = c.gamma;
@@ -447,7 +438,7 @@ attt_status ce_fwd_bwd_run(const attt_bf16 *d_h, const attt_bf16 *d_W, const int
             GemmProblem p{};
             p.a = c.G; p.a_rows_ld = c.Vc; p.a_rows = L; p.a_k = c.Vc;
             p.b = d_W; p.b_rows_ld = d; p.b_rows = d; p.b_k = V;
-            p.M = (int)L; p.N = (int)d; p.K = (int)round_up(Nc, 64); p.BN = kCeBN; p.pair = plan.pair;
+            p.M = (int)L; p.N = (int)d; p.K = (int)round_up(Nc, 64);
             p.b_k_off = (int)v0;
             p.pdl = true;  // E may be rewritten by the chunk kernel: the producer waits
             EpiParams ep{};
@@ -458,7 +449,9 @@ attt_status ce_fwd_bwd_run(const attt_bf16 *d_h, const attt_bf16 *d_W, const int
                 ep.fix_W = reinterpret_cast<const __nv_bfloat16 *>(d_W); ep.fix_ld = d; ep.fix_V = (int)V;
             }
             p.split_ws = c.split_ws; p.split_tick = c.split_tick; p.split_regions = c.split_regions;
-            st = launch_gemm<EPI_F32_ACC, false, true>(p, ep, dev, stream);
+            TilePlan t = plan.dh;
+            if (t.pieces > cdiv(Nc, 64)) t.pieces = (int)cdiv(Nc, 64);  // a short last chunk
+            st = launch_planned<false, false, true>(p, ep, t, dev, stream);
             if (st != ATTT_OK) return st;
         }
     }

@@ -35,6 +35,9 @@ struct GemmProblem {
     float *split_ws = nullptr;
     unsigned int *split_tick = nullptr;
     int split_regions = 0;
+    // EPI_F32_PART: K pieces per tile; piece w (tile-major) stores its 128-row
+    // accumulators at row 128 w (pair: 256 w) of split_ws, BN columns wide.
+    int pieces = 1;
 };
 
 // Pieces per tile for the tiles of a partial last wave: `tiles` tiles over
@@ -58,6 +61,94 @@ inline int tail_pieces(int tiles, int units, int kb_total, int nranks, int regio
     return (1.0 - best) >= 0.1 * waves ? best_s : 1;
 }
 
+// Arguments of the kernel that ends an EPI_F32_PART contraction: out (fp32) =
+// (accumulate ? alpha_m out : 0) + beta_m sum [- gamma_m W[t_m, :]], as
+// EPI_F32_ACC, or out16 (bf16) = alpha sum, as EPI_BF16.  N is a multiple of 4.
+struct SplitReduceArgs {
+    const float *part;
+    int M, N, BN, pieces, rows, tiles_m;  // rows: accumulator rows per tile (128, pair: 256)
+    int64_t ld;
+    float *out;
+    __nv_bfloat16 *out16;
+    float alpha;
+    int accumulate;
+    const float *row_alpha, *row_beta, *row_gamma;
+    const int32_t *fix_tgt;
+    const __nv_bfloat16 *fix_W;
+    int64_t fix_ld;
+    int fix_V;
+};
+attt_status launch_split_reduce(const SplitReduceArgs &a, cudaStream_t stream);
+
+// How a contraction is cut: CTA pairs or single CTAs, the tile width, and the
+// K pieces every tile runs as.
+struct TilePlan {
+    bool pair;
+    int BN, pieces;
+};
+
+// Constants of the plan's estimate, fitted to Eq. 10 calls on GB300 (L 33 to
+// 8,000, every width and both CTA forms): one 64-deep K block takes an SM the
+// time of its MMAs or of its operands from L2, whichever is longer.  Measured
+// per block: 0.33 us for a 256 x 256 pair tile, 0.22 for 256 x 128; single CTAs
+// 0.43-0.47 / 0.35-0.38 / 0.24-0.29 / 0.20 us for the 48 / 40 / 32 / 24 KB of a
+// 128 x 256 / 192 / 128 / 64 tile.  Single CTAs and narrow tiles draw more from
+// L2 per FLOP, so they pay only where they fill idle SMs.
+constexpr int kMaxPieces = 16;
+constexpr double kSmFlops = 12.5e12;                       // bf16 FLOP/s of one SM
+constexpr double kTileFixed = 3e-6, kTileColumn = 1.2e-8;  // ramp of a launch; epilogue of its last tile
+constexpr double kReduceFixed = 3e-6, kReduceByte = 1.6e-13;  // the pieces' reduction (split_reduce.cu)
+constexpr double kTailSum = 1.8e-5;                        // the tail split's partials and their sum
+
+// A K block's operands into one SM: 62 bytes a cycle from L2.
+inline double block_feed_seconds(bool pair, int BN, bool b_mn) {
+    const int cols = !pair ? BN : b_mn ? (int)round_up(BN / 2, 64) : BN / 2;
+    return 9e-9 * (16.0 + cols / 8.0);
+}
+
+// The plan of least estimated time for an M x N result over kb 64-deep K
+// blocks on `sms` SMs.  `regions` bounds the fp32 partials of the K pieces
+// (in 128 x 256 blocks; 0: whole tiles); `tail`: the whole-tile form may cut
+// the tiles of its last wave (tail_pieces).  MN-major B operands (b_mn) come
+// in 64-column boxes, hence the widths.  A width that fills whole waves beats a
+// wider one that does not: 2,048 x 3,584 has 112 tiles of 256 columns for 76
+// pairs (1.47 waves) and 152 of 192 (2.0).  Cutting pays when the tiles leave SMs
+// idle: at 256 rows, d 512, V 8,192 the dh contraction's 2 tiles took 36 us as
+// 4 pieces each and take 6 us as 16 of 128 columns; at 93 rows, d 3,584,
+// V 152,064 its 14 tiles took 337 us as 4 pieces of 4 chunks and take 170 us
+// as 10 pieces of one.
+inline TilePlan plan_tiles(int64_t M, int64_t N, int64_t kb, int sms, int64_t regions, bool tail,
+                           bool b_mn) {
+    TilePlan best{true, 256, 1};
+    double best_t = 1e30;
+    for (int pair = 1; pair >= 0; --pair) {
+        const int64_t rows = pair ? 256 : 128, units = pair ? sms / 2 : sms;
+        for (int BN = 256; BN >= 64; BN -= 64) {
+            if (pair && BN == 64) continue;
+            const int64_t tiles = cdiv(M, rows) * cdiv(N, BN);
+            const double mma = 128.0 * BN * 128 / kSmFlops, feed = block_feed_seconds(pair, BN, b_mn);
+            for (int64_t s = 1; s <= kMaxPieces; ++s) {
+                if (s > 1 && (kb < 16 * s || tiles * s * (rows / 128) * BN > regions * 256)) break;
+                double waves = (double)cdiv(tiles * s, units), extra = 0.0;
+                if (s == 1 && tail) {
+                    const int cut = tail_pieces((int)tiles, (int)units, (int)kb, (int)(rows / 128), (int)regions);
+                    if (cut > 1) {
+                        waves = (double)(tiles / units) + (double)cdiv(tiles % units * cut, units) / cut;
+                        extra = kTailSum;
+                    }
+                }
+                if (s > 1) extra = kReduceFixed + kReduceByte * 8.0 * s * M * N;
+                const double t = waves * cdiv(kb, s) * (mma > feed ? mma : feed) + kTileFixed + BN * kTileColumn + extra;
+                if (t < 0.98 * best_t) {  // the wider and whole forms at equal estimates
+                    best_t = t;
+                    best = TilePlan{pair != 0, BN, (int)s};
+                }
+            }
+        }
+    }
+    return best;
+}
+
 constexpr size_t kMaxSmem = 232448;  // 227 KB opt-in per CTA on sm_100-class parts
 
 inline int gemm_stages(int BN, uint32_t extra = 0) {
@@ -78,7 +169,7 @@ template <int EPI, bool A_MN, bool B_MN>
 attt_status launch_gemm(const GemmProblem &p, const EpiParams &ep, int dev, cudaStream_t stream,
                         int *status = nullptr) {
     if (p.BN < 16 || p.BN > 256 || p.BN % 16 != 0) return ATTT_ERR_INVALID_ARG;
-    if (B_MN && (p.pair ? (p.BN / 2) % 64 : p.BN % 64) != 0) return ATTT_ERR_INVALID_ARG;
+    if (B_MN && p.BN % 64 != 0) return ATTT_ERR_INVALID_ARG;
     if (p.pair && p.BN < 32) return ATTT_ERR_INVALID_ARG;  // BN/2 B rows per CTA (a multiple of 8)
     if (p.M <= 0 || p.N <= 0 || p.K <= 0) return ATTT_ERR_INVALID_ARG;
     CUtensorMap ta, tb;
@@ -127,6 +218,11 @@ attt_status launch_gemm(const GemmProblem &p, const EpiParams &ep, int dev, cuda
     } else if (EPI == EPI_F32_ACC) {
         if (!make_tmap_f32(&tc, ep.out, (uint64_t)p.N, (uint64_t)p.M, (uint64_t)ep.out_ld * 4, 32, 32))
             return ATTT_ERR_INVALID_ARG;
+    } else if (EPI == EPI_F32_PART) {
+        const int64_t t = cdiv(p.M, p.pair ? 256 : 128) * cdiv(p.N, p.BN) * p.pieces * (p.pair ? 2 : 1);
+        if (!p.split_ws || p.pieces < 1 || t * p.BN > (int64_t)p.split_regions * 256) return ATTT_ERR_INVALID_ARG;
+        if (!make_tmap_f32(&tc, p.split_ws, (uint64_t)p.BN, (uint64_t)t * 128, (uint64_t)p.BN * 4, 32, 32))
+            return ATTT_ERR_INVALID_ARG;
     } else if (EPI == EPI_BF16) {
         if (!make_tmap_bf16(&tc, ep.out16, (uint64_t)p.N, (uint64_t)p.M, (uint64_t)ep.out_ld * 2, 32, 32, 64))
             return ATTT_ERR_INVALID_ARG;
@@ -136,9 +232,10 @@ attt_status launch_gemm(const GemmProblem &p, const EpiParams &ep, int dev, cuda
     g.M = p.M;
     g.N = p.N;
     g.BN = p.BN;
-    const int bn_cta = p.pair ? p.BN / 2 : p.BN;  // B rows one CTA stages
+    // B rows one CTA stages (whole 64-column boxes when MN-major)
+    const int bn_cta = !p.pair ? p.BN : B_MN ? (int)round_up(p.BN / 2, 64) : p.BN / 2;
     g.e_stage_bytes = (EPI == EPI_CE_EXP || EPI == EPI_BF16) ? kEStageBytes
-                      : EPI == EPI_F32_ACC                   ? kF32StageBytes
+                      : (EPI == EPI_F32_ACC || EPI == EPI_F32_PART) ? kF32StageBytes
                       : EPI == EPI_KL                        ? kKlXBytes
                                                              : 0u;
     g.stages = gemm_stages(bn_cta, g.e_stage_bytes);
@@ -155,6 +252,10 @@ attt_status launch_gemm(const GemmProblem &p, const EpiParams &ep, int dev, cuda
     g.kb_per_split = g.kb_total;
     g.whole_tiles = tiles;
     g.tail_s = 1;
+    if (EPI == EPI_F32_PART) {
+        g.whole_tiles = 0;
+        g.tail_s = p.pieces;
+    }
     if (EPI == EPI_F32_ACC && p.split_ws && p.split_tick && p.BN % 32 == 0) {
         const int s = tail_pieces(tiles, units, g.kb_total, p.pair ? 2 : 1, p.split_regions);
         if (s > 1) {
@@ -211,6 +312,29 @@ attt_status launch_gemm(const GemmProblem &p, const EpiParams &ep, int dev, cuda
     }
     count_launch();
     return cudaGetLastError() == cudaSuccess ? ATTT_OK : ATTT_ERR_CUDA;
+}
+
+// A contraction with an fp32 (ep.out) or bf16 (ep.out16) result on the tiles of
+// `t`: whole tiles with the fused epilogue, or K pieces and the reduction.
+template <bool OUT16, bool A_MN, bool B_MN>
+attt_status launch_planned(GemmProblem p, const EpiParams &ep, const TilePlan &t, int dev, cudaStream_t stream) {
+    p.pair = t.pair;
+    p.BN = t.BN;
+    if (t.pieces == 1) return launch_gemm<OUT16 ? EPI_BF16 : EPI_F32_ACC, A_MN, B_MN>(p, ep, dev, stream);
+    p.pieces = t.pieces;
+    const attt_status st = launch_gemm<EPI_F32_PART, A_MN, B_MN>(p, ep, dev, stream);
+    if (st != ATTT_OK) return st;
+    SplitReduceArgs a{};
+    a.part = p.split_ws;
+    a.M = p.M; a.N = p.N; a.BN = t.BN; a.pieces = t.pieces; a.rows = t.pair ? 256 : 128;
+    a.tiles_m = (int)cdiv(p.M, a.rows);
+    a.ld = ep.out_ld; a.alpha = ep.alpha;
+    if (OUT16) a.out16 = ep.out16;
+    else a.out = ep.out;
+    a.accumulate = ep.accumulate;
+    a.row_alpha = ep.row_alpha; a.row_beta = ep.row_beta; a.row_gamma = ep.row_gamma;
+    a.fix_tgt = ep.fix_tgt; a.fix_W = ep.fix_W; a.fix_ld = ep.fix_ld; a.fix_V = ep.fix_V;
+    return launch_split_reduce(a, stream);
 }
 
 }  // namespace attt

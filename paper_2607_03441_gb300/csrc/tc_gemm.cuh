@@ -21,7 +21,9 @@
 // When the tiles do not fill the last wave, the tiles of that wave may be
 // cut into K pieces spread over the idle SMs (EPI_F32_ACC): each piece
 // stores an fp32 partial and the last piece to arrive sums them in piece
-// order, so the result does not depend on which piece finishes last.
+// order, so the result does not depend on which piece finishes last.  When
+// all tiles together leave most SMs idle, every tile is cut (EPI_F32_PART)
+// and a second kernel (split_reduce.cu) sums the pieces on every SM.
 #pragma once
 
 #include "attt_common.cuh"
@@ -32,6 +34,7 @@ enum EpiKind : int {
     EPI_CE_EXP = 0,    // per (row, vocab tile): max m, E = exp(z - m) as bf16, sum of E, target logit
     EPI_F32_ACC = 2,   // out[m, n] = (acc ? alpha_m out[m, n] : 0) + beta_m acc [- gamma_m W[t_m, n]]  (fp32)
     EPI_BF16 = 5,      // out16[m, n] = bf16(alpha * acc)  (row-major, through TMA boxes)
+    EPI_F32_PART = 3,  // K piece of every tile: its fp32 accumulator to the piece's region of `out` (split_reduce.cu)
     EPI_KL = 6,        // A tile = 64 rows of A over the same 64 rows of A2: per (row, tile) max, sum of exp, cross term
 };
 
@@ -82,7 +85,8 @@ struct GemmArgs {
     int *status;
     EpiParams ep;
     // Tail split (tc_gemm_kernel / tc_gemm_pair_kernel): tiles [0, whole_tiles)
-    // run whole; every later tile runs as tail_s K pieces.
+    // run whole; every later tile runs as tail_s K pieces.  EPI_F32_PART:
+    // every tile runs as tail_s pieces.
     int whole_tiles, tail_s;
     float *split_ws;           // [tail tile][piece][CTA rank] fp32 partials of 128 x BN, column-quad major
     unsigned int *split_tick;  // [tail tile][CTA rank] arrival counters; 0 between launches
@@ -288,6 +292,31 @@ __device__ __forceinline__ void f32_tile_store(const GemmArgs &g, const CUtensor
         __syncwarp();
         if (lane == 0) {
             tma_store_2d(tm, buf, x, y);
+            bulk_commit();
+        }
+    }
+}
+
+// EPI_F32_PART for this warp's 32 rows: the piece's fp32 accumulator, box by
+// box, to rows [y, y + 32) of the partials' matrix (BN columns wide).  Boxes
+// past the problem's N columns are not stored (never read).
+__device__ __forceinline__ void f32_part_store(const GemmArgs &g, const CUtensorMap *tm, F32Stage &st, int lane, int y,
+                                               int ncols, uint32_t taddr) {
+    for (int c = 0; c < ncols; c += 32, ++st.ec) {
+        const uint32_t buf = st.buf0 + 4096u * (st.ec & 1u);
+        float v[32];
+        tmem_ld_x32(taddr + (uint32_t)c, v);
+        if (lane == 0) bulk_wait_read<1>();  // the store two boxes back has read this box
+        __syncwarp();
+        const uint32_t rowp = buf + (uint32_t)lane * 128u;
+#pragma unroll
+        for (uint32_t q = 0; q < 8; ++q)
+            st_shared_f4(rowp + ((q ^ ((uint32_t)lane & 7u)) << 4),
+                         make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]));
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) {
+            tma_store_2d(tm, buf, c, y);
             bulk_commit();
         }
     }
@@ -736,6 +765,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                                    min(g.N, n_base + g.BN), abort_flag,
                                    [&](int c, float(&v)[32]) { tmem_ld_x32(taddr + (uint32_t)c, v); });
                 }
+            } else if constexpr (EPI == EPI_F32_PART) {
+                if (wi.tm * 128 + 32 * q < g.M)
+                    f32_part_store(g, &tmC, fst, lane, w * 128 + 32 * q, min(g.N - wi.tn * g.BN, g.BN), taddr);
             } else if constexpr (EPI == EPI_BF16) {
                 const int gm = wi.tm * 128 + row;
                 bf16_tile_store(g, &tmC, smem_u32(sE) + (uint32_t)q * 4096u, bec, lane, gm - lane, wi.tn * g.BN,
@@ -748,7 +780,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             if (lane == 0) mbar_arrive(tempty0 + 8 * acc);
         }
         // every TMA store of the epilogue has landed before the CTA retires
-        if constexpr (EPI == EPI_CE_EXP || EPI == EPI_F32_ACC || EPI == EPI_BF16) {
+        if constexpr (EPI != EPI_KL) {
             if (lane == 0) bulk_wait<0>();
         }
     }
@@ -777,8 +809,9 @@ __global__ void __launch_bounds__(kGemmPairThreads, 1)
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int S = g.stages;
-    const int BNh = g.BN / 2;  // B rows held by this CTA
-    const uint32_t b_bytes = gemm_b_stage_bytes(BNh);
+    const int BNh = g.BN / 2;  // B rows of this CTA's half
+    const int b_boxes = (BNh + 63) / 64;  // MN-major: 64-column boxes (BN 192: the second is half used)
+    const uint32_t b_bytes = gemm_b_stage_bytes(B_MN ? 64 * b_boxes : BNh);
     static_assert(EPI != EPI_KL || (!A_MN && !B_MN), "EPI_KL: K-major operands");
     constexpr uint32_t a_bytes = kABytes;
     uint8_t *sA = smem;
@@ -884,7 +917,7 @@ __global__ void __launch_bounds__(kGemmPairThreads, 1)
                     if (!B_MN) {
                         tma_load_2d_pair(b_dst, pb, fb, kbk, brow);
                     } else {
-                        for (int b = 0; b < BNh / 64; ++b) tma_load_2d_pair(b_dst + 8192 * b, pb, fb, brow + 64 * b, kbk);
+                        for (int b = 0; b < b_boxes; ++b) tma_load_2d_pair(b_dst + 8192 * b, pb, fb, brow + 64 * b, kbk);
                     }
                     if (++stage == S) { stage = 0; phase ^= 1u; }
                 }
@@ -980,6 +1013,10 @@ __global__ void __launch_bounds__(kGemmPairThreads, 1)
                                    min(g.N, n_base + g.BN), abort_flag,
                                    [&](int c, float(&v)[32]) { tmem_ld_x32(taddr + (uint32_t)c, v); });
                 }
+            } else if constexpr (EPI == EPI_F32_PART) {
+                if (gm_base + 32 * q < g.M)
+                    f32_part_store(g, &tmC, fst, lane, (w * 2 + (int)rank) * 128 + 32 * q,
+                                   min(g.N - wi.tn * g.BN, g.BN), taddr);
             } else if constexpr (EPI == EPI_BF16) {
                 bf16_tile_store(g, &tmC, smem_u32(sE) + (uint32_t)q * 4096u, bec, lane, gm_base + 32 * q,
                                 wi.tn * g.BN, min(g.N, (wi.tn + 1) * g.BN), taddr);
@@ -991,7 +1028,7 @@ __global__ void __launch_bounds__(kGemmPairThreads, 1)
             if (lane == 0) mbar_arrive_cluster(lead_tempty0 + 8 * acc);
         }
         // every TMA store of the epilogue has landed before the CTA retires
-        if constexpr (EPI == EPI_CE_EXP || EPI == EPI_F32_ACC || EPI == EPI_BF16) {
+        if constexpr (EPI != EPI_KL) {
             if (lane == 0) bulk_wait<0>();
         }
     }

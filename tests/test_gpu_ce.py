@@ -237,6 +237,52 @@ def test_tail_pieces_deterministic(attt, L, V, d):
     assert e < DH_RL2, e
 
 
+@pytest.mark.parametrize("L,V,d", [(1, 8200, 512), (33, 8232, 520), (93, 20000, 3584), (129, 6001, 1288),
+                                   (256, 8192, 512), (300, 20011, 1032), (403, 9000, 3584)])
+def test_every_tile_in_pieces(attt, L, V, d):
+    """Few rows, so every tile of the dh contraction runs as K pieces that a
+    second kernel sums (64- to 256-column tiles, single CTAs and pairs, rows
+    and columns that end inside a tile): every row against the oracle at the
+    tolerances above, and two calls give the same bits."""
+    h = wk.normal_bf16(L + 3, "h", (L, d), 1.0)
+    W = wk.normal_bf16(V + 3, "W", (V, d), 0.05)
+    rng = wk.rng_for(L + V + 3, "t")
+    tgt = rng.integers(0, V, L).astype(np.int32)
+    w = rng.choice(np.array([1.0, 0.5, 0.05], np.float32), L).astype(np.float32)
+    loss, dh, lse = _run(attt, h, W, tgt, w)
+    loss2, dh2, lse2 = _run(attt, h, W, tgt, w)
+    assert loss == loss2
+    np.testing.assert_array_equal(dh.view(np.uint32), dh2.view(np.uint32))
+    np.testing.assert_array_equal(lse.view(np.uint32), lse2.view(np.uint32))
+    rows = np.unique(np.concatenate([[0, L - 1], rng.choice(L, min(L, 12), replace=False)])).astype(np.int64)
+    rlse, _, rdh = oracle.ce_rows(h, W, tgt, w, rows)
+    np.testing.assert_allclose(lse[rows], rlse, atol=LSE_ATOL, rtol=0)
+    assert rel_l2(dh[rows], rdh) < DH_RL2
+
+
+@pytest.mark.parametrize("L,V,d", [(9000, 66000, 16), (60, 9000, 520)])
+def test_reference_jumps_over_chunks_and_narrow_tiles(attt, L, V, d):
+    """Rows far above their reference in the first and the last chunk of a
+    two-chunk call, and in 64-column tiles whose last one ends past the
+    chunk: E rewritten there; those rows against the oracle."""
+    rng = wk.rng_for(78, "jump")
+    h = wk.normal_bf16(78, "h", (L, d), 0.5)
+    W = wk.normal_bf16(78, "W", (V, d), 0.05)
+    hot = [(3, V - 1, 8.0), (17, 30, 8.0), (L - 1, 100, 6.5), (40, V - 70, 6.5)]
+    for j, v, x in hot:
+        h[j] = 0
+        h[j, 0] = wk.bf16_bits(np.array([x], np.float32))[0]
+        W[v, 0] = wk.bf16_bits(np.array([x], np.float32))[0]
+    tgt = rng.integers(0, V, L).astype(np.int32)
+    w = np.ones(L, np.float32)
+    _, dh, lse = _run(attt, h, W, tgt, w)
+    rows = np.array([j for j, _, _ in hot] + [0, 1], np.int64)
+    rlse, _, rdh = oracle.ce_rows(h, W, tgt, w, rows)
+    np.testing.assert_allclose(lse[rows], rlse, atol=LSE_ATOL, rtol=0)
+    for i in range(len(rows)):
+        assert rel_l2(dh[rows[i]], rdh[i]) < DH_RL2, rows[i]
+
+
 def test_launch_counter_counts_every_kernel(attt):
     """One single-chunk call launches the reference kernel, GEMM1, the chunk
     kernel and GEMM2: four kernels, all counted."""
