@@ -353,7 +353,6 @@ attt_status lora_grad_run(const attt_bf16 *d_x, int64_t L, int64_t din, int npro
 
     LoraLayout c = lora_layout(d_ws, L, din, nproj, dout, r);
     const int BN = c.BN;
-
     // prep: adapters to K-major (rank padded with zeros), accumulators zeroed
     {
         PrepArgs a{};
@@ -444,7 +443,8 @@ attt_status lora_grad_run(const attt_bf16 *d_x, int64_t L, int64_t din, int npro
 // and dx are those of the episode's own call.
 // ---------------------------------------------------------------------------
 
-// Split slots of the dx contraction's tail split (as for the CE's dh).
+// Partials of the projection contractions' K pieces, in 128 x 256 fp32 blocks
+// (as for the CE's dh).
 constexpr int kDxSplitRegions = 160;
 
 struct BatchLoraLayout {
@@ -615,11 +615,13 @@ attt_status batch_forward(const attt_bf16 *d_x, const int64_t *off, int E, const
     p.b = d_W0; p.b_rows_ld = d; p.b_rows = d; p.b_k = din;
     p.a2 = c.S; p.a2_rows_ld = c.Ncat; p.a2_rows = R; p.a2_k = c.Ncat;
     p.b2 = c.BT; p.b2_rows_ld = d; p.b2_rows = d; p.b2_k = c.Ncat;
-    p.M = (int)R; p.N = (int)d; p.K = (int)din; p.K2 = (int)c.Ncat; p.BN = 256; p.pair = R > 128;
+    p.M = (int)R; p.N = (int)d; p.K = (int)din; p.K2 = (int)c.Ncat;
     p.pdl = true;
+    p.split_ws = c.split_ws; p.split_regions = kDxSplitRegions;
     EpiParams ep{};
     ep.out16 = reinterpret_cast<__nv_bfloat16 *>(d_h); ep.out_ld = d; ep.alpha = 1.0f;
-    return launch_gemm<EPI_BF16, false, true>(p, ep, dev, stream);
+    const TilePlan t = plan_tiles(R, d, cdiv(din, 64) + cdiv(c.Ncat, 64), num_sms(dev), kDxSplitRegions, false, true);
+    return launch_planned<true, false, true>(p, ep, t, dev, stream);
 }
 
 attt_status batch_grads(const attt_bf16 *d_x, const attt_bf16 *d_dy, const int64_t *off, int E, int64_t din,
@@ -708,12 +710,13 @@ attt_status batch_input_grad(const attt_bf16 *d_dy, const int64_t *off, int E, c
     p.b = d_W0; p.b_rows_ld = d; p.b_rows = din; p.b_k = d;
     p.a2 = c.S; p.a2_rows_ld = c.Ncat; p.a2_rows = R; p.a2_k = c.Ncat;
     p.b2 = c.ACAT; p.b2_rows_ld = c.Ncat; p.b2_rows = din; p.b2_k = c.Ncat;
-    p.M = (int)R; p.N = (int)din; p.K = (int)d; p.K2 = (int)c.Ncat; p.BN = 256; p.pair = R > 128;
+    p.M = (int)R; p.N = (int)din; p.K = (int)d; p.K2 = (int)c.Ncat;
     p.pdl = true;
     p.split_ws = c.split_ws; p.split_tick = c.tickets + c.tiles; p.split_regions = kDxSplitRegions;
     EpiParams ep{};
     ep.out = d_dx; ep.out_ld = din; ep.accumulate = 0; ep.alpha = 1.0f;
-    return launch_gemm<EPI_F32_ACC, false, false>(p, ep, dev, stream);
+    const TilePlan t = plan_tiles(R, din, cdiv(d, 64) + cdiv(c.Ncat, 64), num_sms(dev), kDxSplitRegions, true, false);
+    return launch_planned<false, false, false>(p, ep, t, dev, stream);
 }
 
 // ---------------------------------------------------------------------------
@@ -727,7 +730,7 @@ struct ProjLayout {
     __nv_bfloat16 *s16;      // s u or s v, [L, rpad] bf16 row-major
     unsigned int *tickets;   // the skinny launch's tiles, then the tail split's counters
     float *part;             // the skinny launch's partial slots
-    float *split_ws;         // input gradient: tail-split partials
+    float *split_ws;         // partials of the contraction's K pieces
     int64_t tiles;
     size_t bytes;
 };
@@ -744,7 +747,7 @@ static ProjLayout proj_layout(void *ws, int64_t L, int64_t din, int64_t dout, in
     c.s16 = cv.take<__nv_bfloat16>((size_t)(L * c.rpad));
     c.tickets = cv.take<unsigned int>((size_t)(c.tiles + kDxSplitRegions));
     c.part = cv.take<float>((size_t)(c.tiles + kGroupMaxGrid) * 128 * c.rpad);
-    if (!fwd) c.split_ws = cv.take<float>((size_t)kDxSplitRegions * 128 * 256);
+    c.split_ws = cv.take<float>((size_t)kDxSplitRegions * 128 * 256);
     c.bytes = (size_t)round_up((int64_t)cv.used, 256);
     return c;
 }
@@ -814,11 +817,14 @@ attt_status attt_lora_forward(const attt_bf16 *d_x, const attt_bf16 *d_W0, const
         p.b = d_W0; p.b_rows_ld = dout; p.b_rows = dout; p.b_k = din;
         p.a2 = c.s16; p.a2_rows_ld = c.rpad; p.a2_rows = L; p.a2_k = c.rpad;
         p.b2 = d_B; p.b2_rows_ld = dout; p.b2_rows = dout; p.b2_k = r;
-        p.M = (int)L; p.N = (int)dout; p.K = (int)din; p.K2 = c.rpad; p.BN = 256; p.pair = L > 128;
+        p.M = (int)L; p.N = (int)dout; p.K = (int)din; p.K2 = c.rpad;
         p.pdl = true;
+        p.split_ws = c.split_ws; p.split_regions = kDxSplitRegions;
         EpiParams ep{};
         ep.out16 = reinterpret_cast<__nv_bfloat16 *>(d_h); ep.out_ld = dout; ep.alpha = 1.0f;
-        st = launch_gemm<EPI_BF16, false, true>(p, ep, dev, stream);
+        const TilePlan t = plan_tiles(L, dout, cdiv(din, 64) + cdiv(c.rpad, 64), num_sms(dev), kDxSplitRegions, false,
+                                      true);
+        st = launch_planned<true, false, true>(p, ep, t, dev, stream);
         if (st != ATTT_OK) return st;
     }
     return ATTT_OK;
@@ -856,12 +862,14 @@ attt_status attt_lora_input_grad(const attt_bf16 *d_dy, const attt_bf16 *d_W0, c
         p.b = d_W0; p.b_rows_ld = dout; p.b_rows = din; p.b_k = dout;
         p.a2 = c.s16; p.a2_rows_ld = c.rpad; p.a2_rows = L; p.a2_k = c.rpad;
         p.b2 = d_A; p.b2_rows_ld = r; p.b2_rows = din; p.b2_k = r;
-        p.M = (int)L; p.N = (int)din; p.K = (int)dout; p.K2 = c.rpad; p.BN = 256; p.pair = L > 128;
+        p.M = (int)L; p.N = (int)din; p.K = (int)dout; p.K2 = c.rpad;
         p.pdl = true;
         p.split_ws = c.split_ws; p.split_tick = c.tickets + c.tiles; p.split_regions = kDxSplitRegions;
         EpiParams ep{};
         ep.out = d_dx; ep.out_ld = din; ep.accumulate = 0; ep.alpha = 1.0f;
-        st = launch_gemm<EPI_F32_ACC, false, false>(p, ep, dev, stream);
+        const TilePlan t = plan_tiles(L, din, cdiv(dout, 64) + cdiv(c.rpad, 64), num_sms(dev), kDxSplitRegions, true,
+                                      false);
+        st = launch_planned<false, false, false>(p, ep, t, dev, stream);
         if (st != ATTT_OK) return st;
     }
     return ATTT_OK;

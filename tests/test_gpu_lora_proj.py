@@ -107,3 +107,25 @@ def test_launch_counts_and_arguments(attt):
         attt.attt_lora_forward(torch.zeros(L, 36, dtype=torch.bfloat16, device=DEV),
                                torch.zeros(36, dout, dtype=torch.bfloat16, device=DEV),
                                torch.zeros(36, r, dtype=torch.bfloat16, device=DEV), Bd, 1.0)
+
+
+@pytest.mark.parametrize("shape", [(93, 3584, 1048, 16), (200, 4096, 3584, 8), (300, 2056, 3592, 64),
+                                   (403, 1544, 2056, 16), (1800, 1024, 3584, 16), (2048, 584, 3592, 32)])
+def test_planned_tiles(attt, shape):
+    """Shapes whose contractions run on each form of the tile plan: K pieces
+    summed by a second kernel (bf16 and fp32 results), 192-column pair tiles
+    (an MN-major operand in half-used boxes) and narrow tiles, with rows and
+    columns that end inside a tile: both directions on sampled rows at the
+    tolerances above, and two calls give the same bits."""
+    L, din, dout, r = shape
+    x, dy, W0, A, B = _inputs(L + din + dout, L, din, dout, r)
+    s = 2.0
+    w = (bf16_dev(W0), bf16_dev(A), bf16_dev(B), s)
+    rows = _rows(L, 20, L)
+    h = attt.attt_lora_forward(bf16_dev(x), *w)
+    assert torch.equal(h, attt.attt_lora_forward(bf16_dev(x), *w))
+    assert rel_l2(h.float().cpu().numpy()[rows], oracle.lora_forward(x[rows], W0, A, B, s)) < H_RL2
+    dx = attt.attt_lora_input_grad(bf16_dev(dy), *w)
+    assert torch.equal(dx, attt.attt_lora_input_grad(bf16_dev(dy), *w))
+    assert rel_l2(dx.cpu().numpy()[rows], oracle.lora_input_grad(dy[rows], W0, A, B, s)) < DX_RL2
+    assert attt.attt_device_status() == 0
