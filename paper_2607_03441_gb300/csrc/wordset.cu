@@ -29,6 +29,9 @@
 
 namespace {
 
+using attt::griddep_launch_dependents;
+using attt::griddep_wait;
+
 constexpr int kMaxUpdates = 4096;
 constexpr int kProbeLimit = 1 << 20;
 constexpr int kInsThreads = 256;
@@ -87,42 +90,88 @@ struct RepArgs {
 };
 
 constexpr int kChunk = 2048;                 // largest text chunk of a block iteration
+constexpr int kStageTail = 64;               // bytes past the chunk staged with it (words that cross its end)
 constexpr int kChunkWords = kChunk / 2 + 1;  // a word start follows whitespace
 constexpr int kLocalSlots = 2048;            // block-local word table (>= 2 x kChunkWords)
 
-// Hashes the word at chunk offset `off` (FNV-1a 64 over its bytes, then a
-// 64-bit finalizer), drops it if it repeats an earlier word of the chunk
-// (block-local table of 64-bit shared-memory keys: hash tag | offset + 1),
-// else claims or finds its slot in the episode's index and sets update k's
-// bit.  Returns the slot's mask words if this thread set the bit first (it
-// owns the word's element of W(x_k)), with the previous value of mask word
-// k / 64 in *old; nullptr otherwise.
-__device__ __forceinline__ const unsigned long long *record_word(const RepArgs &a, const TextView &v, int64_t c0,
-                                                                 uint32_t off, unsigned long long *s_key, int kw,
-                                                                 unsigned long long kbit, unsigned long long *old) {
-    const int64_t p = a.base + c0 + off;
-    unsigned long long h = 0xcbf29ce484222325ull;
-    int64_t e = p;
-    for (unsigned int ch = v.at(e); !is_space(ch); ch = v.at(++e)) h = (h ^ ch) * 0x100000001b3ull;
-    const int64_t len = e - p;
-    h = finalize64(h);
-    const unsigned long long lkey = (h & 0xFFFFFFFF00000000ull) | (unsigned long long)(off + 1u);
-    unsigned int li = (unsigned int)(h >> 20) & (kLocalSlots - 1);
+// The block's chunk of the current text in shared memory: byte off of the
+// chunk, from the staged bytes or (a word that runs past them) the text.
+struct ChunkView {
+    const uint8_t *staged;  // [chunk + kStageTail], spaces past the text
+    int nstaged;
+    const uint8_t *text;  // the whole text
+    int64_t c0, n;
+    __device__ __forceinline__ unsigned int at(int64_t off) const {
+        return off < nstaged ? (unsigned int)staged[off] : (c0 + off < n ? (unsigned int)text[c0 + off] : 0x20u);
+    }
+};
+
+// A word of the chunk: its hash and length, and whether it is the first
+// occurrence in the chunk (FNV-1a 64 over its bytes, then a 64-bit finalizer;
+// the block-local table holds 64-bit keys hash tag | offset + 1).
+struct Word {
+    unsigned long long h;
+    int64_t len;
+    bool first;
+};
+
+__device__ __forceinline__ Word local_word(const ChunkView &c, uint32_t off, unsigned long long *s_key) {
+    Word w{0xcbf29ce484222325ull, 0, true};
+    for (unsigned int ch = c.at(off); !is_space(ch); ch = c.at(off + ++w.len)) w.h = (w.h ^ ch) * 0x100000001b3ull;
+    w.h = finalize64(w.h);
+    const unsigned long long lkey = (w.h & 0xFFFFFFFF00000000ull) | (unsigned long long)(off + 1u);
+    unsigned int li = (unsigned int)(w.h >> 20) & (kLocalSlots - 1);
     for (int probe = 0; probe < kLocalSlots; ++probe, li = (li + 1) & (kLocalSlots - 1)) {
         const unsigned long long o = atomicCAS(&s_key[li], 0ull, lkey);
         if (o == 0ull) break;
-        if ((o >> 32) == (lkey >> 32) && word_equal(v, a.base + c0 + (int64_t)(o & 0xFFFFFFFFull) - 1, p))
-            return nullptr;  // repeats a word of this chunk
+        if ((o >> 32) != (lkey >> 32)) continue;
+        const int64_t oo = (int64_t)(o & 0xFFFFFFFFull) - 1;  // the earlier word's offset
+        bool same = is_space(c.at(oo + w.len));
+        for (int64_t i = 0; same && i < w.len; ++i) same = c.at(oo + i) == c.at(off + i);
+        if (same) {
+            w.first = false;  // repeats a word of this chunk
+            break;
+        }
     }
-    const unsigned long long key = (h & 0xFFFF000000000000ull) |
-                                   ((unsigned long long)(len < 0xFFFF ? len : 0xFFFF) << 32) |
-                                   (unsigned long long)(p + 1);
-    unsigned long long idx = h & a.cap_mask;
+    return w;
+}
+
+// The word at chunk offset off (length len) against the word at position a of
+// the episode's texts whose key has the same length field: below 0xFFFF that
+// is the length, and the bytes are compared eight loads at a time (one round
+// trip to the arena for most words, where a byte loop takes one per byte).
+__device__ __forceinline__ bool same_word(const TextView &v, const ChunkView &c, int64_t a, uint32_t off, int64_t len) {
+    if (len >= 0xFFFF) return word_equal(v, a, v.base + c.c0 + off);
+    const uint8_t *pa = a < v.base ? v.arena + a : v.text + (a - v.base);
+    for (int64_t i = 0; i < len; i += 8) {
+        unsigned int x[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) x[j] = i + j < len ? (unsigned int)pa[i + j] : 0u;
+        bool same = true;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) same = same && (i + j >= len || x[j] == c.at(off + i + j));
+        if (!same) return false;
+    }
+    return true;
+}
+
+// Claims or finds the word's slot in the episode's index and sets update k's
+// bit.  Returns the slot's mask words if this thread set the bit first (it
+// owns the word's element of W(x_k)), with the previous value of mask word
+// k / 64 in *old; nullptr otherwise.
+__device__ __forceinline__ const unsigned long long *record_word(const RepArgs &a, const TextView &v,
+                                                                 const ChunkView &c, uint32_t off, const Word &w,
+                                                                 int kw, unsigned long long kbit,
+                                                                 unsigned long long *old) {
+    const unsigned long long key = (w.h & 0xFFFF000000000000ull) |
+                                   ((unsigned long long)(w.len < 0xFFFF ? w.len : 0xFFFF) << 32) |
+                                   (unsigned long long)(a.base + c.c0 + off + 1);
+    unsigned long long idx = w.h & a.cap_mask;
     for (int probe = 0; probe < kProbeLimit; ++probe) {
         const unsigned long long k0 = atomicCAS(a.keys + idx, 0ull, key);
         if (k0 == 0ull || ((k0 >> 32) == (key >> 32) &&
                            ATTT_GUARD((int64_t)(k0 & 0xFFFFFFFFull) - 1 < a.base + a.n, a.status) &&
-                           word_equal(v, (int64_t)(k0 & 0xFFFFFFFFull) - 1, p))) {
+                           same_word(v, c, (int64_t)(k0 & 0xFFFFFFFFull) - 1, off, w.len))) {
             unsigned long long *m = a.masks + (size_t)idx * a.W;
             *old = atomicOr(m + kw, kbit);
             return (*old & kbit) ? nullptr : m;  // else another block owns it
@@ -137,50 +186,61 @@ __device__ __forceinline__ const unsigned long long *record_word(const RepArgs &
 // in the index and counts |W(x_k)| and |W(x_k) & W(x_i)|; the last block to
 // finish applies Eq. 6 / Eq. 7 and the filter.
 //
-// Each block takes chunks of 256 to 2,048 bytes of the text.  Word starts go to a list
-// in shared memory; each word goes through record_word (a word repeated
-// inside the chunk costs one global probe instead of one per occurrence: Zipf
-// text repeats its frequent words many times per chunk).  The owners of
-// words of W(x_k) add one to |W(x_k) & W(x_i)| for every earlier update i
-// whose bit their mask has: one warp ballot per bit set in any lane, added by
-// one lane into a shared-memory histogram per block, flushed once.
+// Each block takes chunks of 256 to 2,048 bytes of the text, staged in shared
+// memory.  Word starts go to a list; each word is hashed and dropped if the
+// chunk has it already (local_word: Zipf text repeats its frequent words many
+// times per chunk), else it goes through record_word.  The owners of words of
+// W(x_k) add one to |W(x_k) & W(x_i)| for every earlier update i whose bit
+// their mask has: one warp ballot per bit set in any lane, added by one lane
+// into a shared-memory histogram per block, flushed once.
+//
+// What bounds it is latency: a text is a chain of round trips (text, slot
+// claim, byte compare, mask, counters, ticket), not bytes.  So consecutive
+// texts' kernels are launched as programmatic dependents: the next one's
+// blocks are resident with their tables cleared when this one completes.  They
+// read nothing, the caller's text included, before griddep_wait.
 __global__ void __launch_bounds__(kInsThreads) repetition_kernel(RepArgs a) {
     extern __shared__ unsigned int s_inter[];  // [k]
     __shared__ unsigned long long s_key[kLocalSlots];
     __shared__ uint32_t s_start[kChunkWords];
+    __shared__ uint8_t s_text[kChunk + kStageTail];
     __shared__ unsigned int s_nstart, s_distinct;
     __shared__ float s_max[kInsThreads / 32];
     __shared__ int s_last;
     const TextView v{a.arena, a.text, a.base, a.n};
     for (int i = threadIdx.x; i < a.k; i += blockDim.x) s_inter[i] = 0u;
-    if (threadIdx.x == 0) s_distinct = 0u;
+    for (int i = threadIdx.x; i < kLocalSlots; i += blockDim.x) s_key[i] = 0ull;
+    if (threadIdx.x == 0) s_distinct = s_nstart = 0u;
+    griddep_launch_dependents();
+    griddep_wait();
 
     const int kw = a.k >> 6;
     const unsigned long long kbit = 1ull << (a.k & 63);
     for (int64_t c0 = (int64_t)blockIdx.x * a.chunk; c0 < a.n; c0 += (int64_t)gridDim.x * a.chunk) {
-        for (int i = threadIdx.x; i < kLocalSlots; i += blockDim.x) s_key[i] = 0ull;
-        if (threadIdx.x == 0) s_nstart = 0u;
-        __syncthreads();
         const int cn = (int)(a.n - c0 < a.chunk ? a.n - c0 : a.chunk);
+        for (int i = threadIdx.x; i < a.chunk + kStageTail; i += blockDim.x)
+            s_text[i] = c0 + i < a.n ? a.text[c0 + i] : (uint8_t)0x20;
+        const unsigned int before = (threadIdx.x == 0 && c0 > 0) ? (unsigned int)a.text[c0 - 1] : 0x20u;
+        __syncthreads();
         for (int i = threadIdx.x; i < cn; i += blockDim.x) {
-            const int64_t off = c0 + i;
-            const unsigned int b = a.text[off];
-            a.arena[a.base + off] = (uint8_t)b;
-            const unsigned int prev = off == 0 ? 0x20u : (unsigned int)a.text[off - 1];
-            if (!is_space(b) && is_space(prev)) s_start[atomicAdd(&s_nstart, 1u)] = (uint32_t)i;
+            const unsigned int prev = i == 0 ? before : (unsigned int)s_text[i - 1];
+            if (!is_space(s_text[i]) && is_space(prev)) s_start[atomicAdd(&s_nstart, 1u)] = (uint32_t)i;
         }
         __syncthreads();
+        const ChunkView cv{s_text, a.chunk + kStageTail, a.text, c0, a.n};
         const int ns = (int)s_nstart;
         // rounds of blockDim.x words, so that whole warps reach the counting
         // step together
         for (int w0 = 0; w0 < ns; w0 += blockDim.x) {
             const int w = w0 + threadIdx.x;
+            Word word{0ull, 0, false};
+            if (w < ns) word = local_word(cv, s_start[w], s_key);
             const unsigned long long *m = nullptr;  // this lane's word of x_k, if it owns one
             unsigned long long old = 0ull;
-            if (w < ns) m = record_word(a, v, c0, s_start[w], s_key, kw, kbit, &old);
+            if (word.first) m = record_word(a, v, cv, s_start[w], word, kw, kbit, &old);
             const bool own = m != nullptr;
-            if (own) atomicAdd(&s_distinct, 1u);
-            __syncwarp();
+            const unsigned int owners = __popc(__ballot_sync(0xffffffffu, own));
+            if ((threadIdx.x & 31) == 0 && owners) atomicAdd(&s_distinct, owners);
             // |W(x_k) & W(x_i)| += number of owned words whose mask has bit i:
             // per mask word, one ballot per bit set in any lane
             for (int j = 0; j <= kw; ++j) {
@@ -202,18 +262,24 @@ __global__ void __launch_bounds__(kInsThreads) repetition_kernel(RepArgs a) {
                 }
             }
         }
+        for (int i = threadIdx.x; i < cn; i += blockDim.x) a.arena[a.base + c0 + i] = s_text[i];
+        __syncthreads();
+        if (c0 + (int64_t)gridDim.x * a.chunk >= a.n) break;
+        for (int i = threadIdx.x; i < kLocalSlots; i += blockDim.x) s_key[i] = 0ull;
+        if (threadIdx.x == 0) s_nstart = 0u;
         __syncthreads();
     }
-    __syncthreads();
     for (int i = threadIdx.x; i < a.k; i += blockDim.x)
         if (s_inter[i]) atomicAdd(a.inter + i, s_inter[i]);
     if (threadIdx.x == 0 && s_distinct) atomicAdd(a.distinct, s_distinct);
-    __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(a.ticket, 1u) == gridDim.x - 1;
+    if (threadIdx.x == 0) {
+        __threadfence();  // the block's counts (ordered before by the barrier) precede its ticket
+        s_last = atomicAdd(a.ticket, 1u) == gridDim.x - 1;
+        __threadfence();
+    }
     __syncthreads();
     if (!s_last) return;
-    __threadfence();
 
     // Eq. 6 / Eq. 7 and the filter; clears the counters for the next update
     const unsigned int dk = __ldcg(a.distinct);
@@ -353,7 +419,17 @@ attt_status attt_repetition(attt_wordsets *s, const uint8_t *d_text, int64_t nby
     int64_t blocks = cdiv(nbytes, a.chunk);
     if (blocks > sms * 4) blocks = sms * 4;
     if (blocks < 1) blocks = 1;
-    repetition_kernel<<<(unsigned)blocks, kInsThreads, (size_t)a.k * sizeof(unsigned int), stream>>>(a);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(kInsThreads);
+    cfg.dynamicSmemBytes = (size_t)a.k * sizeof(unsigned int);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, repetition_kernel, a) != cudaSuccess) return ATTT_ERR_CUDA;
     count_launch();
     if (cudaGetLastError() != cudaSuccess) return ATTT_ERR_CUDA;
     s->count = a.k + 1;
