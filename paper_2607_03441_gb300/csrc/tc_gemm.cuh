@@ -637,7 +637,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     const int nwork = work_count(g, g.tiles_m);
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             // ---------------- TMA producer ----------------
             if (!g.operands_ready) griddep_wait();
             int stage = 0;
@@ -689,13 +689,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             // ---------------- MMA issuer ----------------
             const uint32_t idesc = idesc_bf16_f32((uint32_t)g.BN, A_MN, B_MN);
             int stage = 0;
             uint32_t phase = 0;
             int it = 0;
-            bool ok = true;
+            bool ok = true, ready = false;
             for (int w = blockIdx.x; w < nwork && ok; w += gridDim.x, ++it) {
                 const Work wi = work_item(g, w, g.tiles_m);
                 const int kb0 = wi.kb0, kb1 = wi.kb1;
@@ -704,8 +704,12 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(acc * g.BN);
                 for (int kb = kb0; kb < kb1; ++kb) {
-                    if (!mbar_wait(full0 + 8 * stage, phase, abort_flag)) { ok = false; break; }
+                    if (!ready && !mbar_wait(full0 + 8 * stage, phase, abort_flag)) { ok = false; break; }
                     tc_fence_after();
+                    // the next stage's barrier is read while this stage's MMAs issue
+                    const int next = stage + 1 == S ? 0 : stage + 1;
+                    const uint32_t next_phase = next == 0 ? phase ^ 1u : phase;
+                    ready = mbar_test_wait(full0 + 8 * next, next_phase);
                     const uint32_t a_addr = smem_u32(sA + (size_t)stage * kABytes);
                     const uint32_t b_addr = smem_u32(sB + (size_t)stage * b_bytes);
 #pragma unroll
@@ -717,7 +721,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                         umma_bf16(d_tmem, ad, bd, idesc, (kb > kb0 || kk > 0) ? 1u : 0u);
                     }
                     umma_commit(empty0 + 8 * stage);
-                    if (++stage == S) { stage = 0; phase ^= 1u; }
+                    stage = next;
+                    phase = next_phase;
                 }
                 if (!ok) break;
                 umma_commit(tfull0 + 8 * acc);
@@ -869,7 +874,7 @@ __global__ void __launch_bounds__(kGemmPairThreads, 1)
     const uint32_t lead_tempty0 = mapa_shared(tempty0, 0);
 
     if (warp == 0 || warp == 6) {
-        if (lane == 0) {
+        if (elect_one()) {
             // ---------------- TMA producers (both CTAs; warp 0 even, warp 6 odd stages) ----------------
             if (!g.operands_ready) griddep_wait();
             const uint32_t pid = warp == 0 ? 0u : 1u;  // this producer's stages: pos % 2 == pid
@@ -934,13 +939,13 @@ __global__ void __launch_bounds__(kGemmPairThreads, 1)
             }
         }
     } else if (warp == 1) {
-        if (lane == 0 && leader) {
+        if (leader && elect_one()) {
             // ---------------- MMA issuer (even CTA) ----------------
             const uint32_t idesc = idesc_bf16_f32((uint32_t)g.BN, A_MN, B_MN, 256);
             int stage = 0;
             uint32_t phase = 0;
             int it = 0;
-            bool ok = true;
+            bool ok = true, ready = false;
             for (int w = cid; w < nwork && ok; w += ncl, ++it) {
                 const Work wi = work_item(g, w, tiles_m2);
                 const int kb0 = wi.kb0, kb1 = wi.kb1;
@@ -949,8 +954,12 @@ __global__ void __launch_bounds__(kGemmPairThreads, 1)
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(acc * g.BN);
                 for (int kb = kb0; kb < kb1; ++kb) {
-                    if (!mbar_wait(full0 + 8 * stage, phase, abort_flag)) { ok = false; break; }
+                    if (!ready && !mbar_wait(full0 + 8 * stage, phase, abort_flag)) { ok = false; break; }
                     tc_fence_after();
+                    // the next stage's barrier is read while this stage's MMAs issue
+                    const int next = stage + 1 == S ? 0 : stage + 1;
+                    const uint32_t next_phase = next == 0 ? phase ^ 1u : phase;
+                    ready = mbar_test_wait(full0 + 8 * next, next_phase);
                     const uint32_t a_addr = smem_u32(sA + (size_t)stage * a_bytes);
                     const uint32_t b_addr = smem_u32(sB + (size_t)stage * b_bytes);
 #pragma unroll
@@ -962,7 +971,8 @@ __global__ void __launch_bounds__(kGemmPairThreads, 1)
                         umma_bf16_pair(d_tmem, ad, bd, idesc, (kb > kb0 || kk > 0) ? 1u : 0u);
                     }
                     umma_commit_pair(empty0 + 8 * stage, 3);
-                    if (++stage == S) { stage = 0; phase ^= 1u; }
+                    stage = next;
+                    phase = next_phase;
                 }
                 if (!ok) break;
                 umma_commit_pair(tfull0 + 8 * acc, 3);

@@ -342,7 +342,7 @@ __global__ void __launch_bounds__(kGroupThreads, 1)
     const int64_t x1 = ((int64_t)blockIdx.x + 1) * g.total_stages / G;
 
     if (warp == 0 || warp == 6) {
-        if (lane == 0) {
+        if (elect_one()) {
             griddep_wait();  // the B operands (adapters, u, v) come from the previous grid
             const uint32_t pid = warp == 0 ? 0u : 1u;  // this producer's stages: pos % 2 == pid
             uint32_t pos = 0;
@@ -398,12 +398,12 @@ __global__ void __launch_bounds__(kGroupThreads, 1)
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t idesc = idesc_bf16_f32((uint32_t)g.BN, A_MN, B_MN);
             int stage = 0;
             uint32_t phase = 0;
             int it = 0;
-            bool ok = true;
+            bool ok = true, ready = false;
             GroupSeg sg;
             for (int64_t x = x0; ok && group_next(g, x, x1, sg); ++it) {
                 const int kb0 = sg.kb0, kb1 = sg.kb1;
@@ -412,8 +412,12 @@ __global__ void __launch_bounds__(kGroupThreads, 1)
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(acc * g.BN);
                 for (int kb = kb0; kb < kb1; kb += KBS) {
-                    if (!mbar_wait(full0 + 8 * stage, phase, abort_flag)) { ok = false; break; }
+                    if (!ready && !mbar_wait(full0 + 8 * stage, phase, abort_flag)) { ok = false; break; }
                     tc_fence_after();
+                    // the next stage's barrier is read while this stage's MMAs issue
+                    const int next = stage + 1 == S ? 0 : stage + 1;
+                    const uint32_t next_phase = next == 0 ? phase ^ 1u : phase;
+                    ready = mbar_test_wait(full0 + 8 * next, next_phase);
                     for (int j = 0; j < KBS; ++j) {
                         const uint32_t a_addr = smem_u32(sA + (size_t)stage * kABytesS + (size_t)j * a1);
                         const uint32_t b_addr = smem_u32(sB + (size_t)stage * b_bytes + (size_t)j * b1);
@@ -427,7 +431,8 @@ __global__ void __launch_bounds__(kGroupThreads, 1)
                         }
                     }
                     umma_commit(empty0 + 8 * stage);
-                    if (++stage == S) { stage = 0; phase ^= 1u; }
+                    stage = next;
+                    phase = next_phase;
                 }
                 if (!ok) break;
                 umma_commit(tfull0 + 8 * acc);
