@@ -20,10 +20,12 @@
 // dx = dy W0^T + s (dy B^T) A^T.  Each is one tcgen05 contraction whose K runs
 // over two operand pairs, [x | s u] [W0 ; B] and [dy | s v] [W0^T ; A^T], after
 // a skinny grouped launch that forms s u = s x A or s v = s dy B^T in bf16.
+#include <atomic>
 #include <cmath>
 
 #include "gemm_launch.cuh"
 #include "tc_group.cuh"
+#include "tc_skinny.cuh"
 
 namespace attt {
 
@@ -229,6 +231,11 @@ struct GroupSpec {
     float *outp[kMaxProj];
 };
 
+// Limits of the skinny form (tc_skinny.cuh): ring slots, projections (a slot
+// holds a 64-column box per adapter) and columns.
+constexpr int kSkinnyMaxStages = 12, kSkinnyMaxProj = 4, kSkinnyMaxCols = 192;
+constexpr int kSkinnyMinBlocks = 8;
+constexpr double kSkinnyExtra = 5.0;  // microseconds (skinny_grad_plan)
 constexpr int kGroupMinStages = 2;
 // Ring stages a grouped launch's shared-memory ring keeps when it can (the
 // stage shape: the most K blocks per stage that leaves this many).  Measured
@@ -331,6 +338,291 @@ static attt_status launch_group(const GroupSpec *specs, int n, int BN, float *pa
     return cudaGetLastError() == cudaSuccess ? ATTT_OK : ATTT_ERR_CUDA;
 }
 
+// ---------------------------------------------------------------------------
+// Skinny launches (tc_skinny.cuh)
+// ---------------------------------------------------------------------------
+
+// Clusters of c CTAs (1 <= c <= kSkinnyMaxCluster) of the skinny kernel that
+// the device holds at once, one CTA per SM: fewer than SMs / c, since a cluster
+// lies within one GPC (a GB300 holds 152, 76, 46, 36, 28, 23, 15, 15; the 16
+// row tiles of 2,048 rows on clusters of 8 ran as two waves, 18 us against 9).
+static int skinny_clusters(int c, int dev) {
+    static std::atomic<int> held[16][kSkinnyMaxCluster + 1];  // 0: not asked yet
+    const bool cached = dev >= 0 && dev < 16;
+    int n = cached ? held[dev][c].load(std::memory_order_relaxed) : 0;
+    if (n == 0) {
+        const int sms = num_sms(dev);
+        n = sms / c > 0 ? sms / c : 1;
+        auto kern = tc_skinny_kernel<false>;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(c * n));
+        cfg.blockDim = dim3(kSkinnyThreads);
+        cfg.dynamicSmemBytes = kMaxSmem;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)c;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int m = 0;
+        if (set_smem_limit(reinterpret_cast<const void *>(kern), kMaxSmem, dev) &&
+            cudaOccupancyMaxActiveClusters(&m, kern, &cfg) == cudaSuccess && m > 0 && m < n)
+            n = m;
+        if (cached) held[dev][c].store(n, std::memory_order_relaxed);
+    }
+    return n;
+}
+
+// Microseconds one K block takes a CTA: its operands from L2 (62 bytes a cycle
+// into an SM) or the issue of its loads and MMAs, whichever is longer.
+static double skinny_block(int nb, int n, bool mn) {
+    const double feed = 0.009 * (16.0 + (mn ? 8.0 * nb : n / 8.0)), issue = 0.06 + 0.06 * nb;
+    return feed > issue ? feed : issue;
+}
+
+// The most CTAs per tile (at most one per K block) with which `tiles` clusters
+// are resident together; 0 if the tiles alone are not.
+static int skinny_cluster(int64_t tiles, int64_t kb, int dev) {
+    int c = kSkinnyMaxCluster < kb ? kSkinnyMaxCluster : (int)kb;
+    while (c > 0 && tiles > skinny_clusters(c, dev)) --c;
+    return c;
+}
+
+// Launches the groups of g (its groups, segments, tiles and columns filled in)
+// on `clusters` clusters of `c` CTAs.  `pdl`: a programmatic dependent of the
+// previous kernel.  False in *fits (nothing launched) if the accumulators of a
+// tile exceed TMEM or shared memory.
+template <bool A_MN>
+static attt_status launch_skinny(const SkinnyMaps &maps, SkinnyArgs &g, int64_t clusters, int c, bool pdl, int dev,
+                                 cudaStream_t stream) {
+    uint32_t stage = 0;
+    int ncols = 0, kb = 0;  // columns and K blocks of one CTA at most
+    for (int q = 0; q < g.ngroup; ++q) {
+        const SkinnyGroup &gr = g.grp[q];
+        if (gr.ncols > ncols) ncols = gr.ncols;
+        if (cdiv(gr.kb_total, gr.split) > kb) kb = (int)cdiv(gr.kb_total, gr.split);
+        for (int i = gr.seg0; i < gr.seg0 + gr.nseg; ++i) {
+            const SkinnySeg &s = g.seg[i];
+            const uint32_t b = kABytes + (uint32_t)s.nb * (s.b_mn ? 8192u : (uint32_t)s.n * 128u);
+            if (b > stage) stage = b;
+        }
+    }
+    const uint32_t bound = (uint32_t)kMaxSmem - 2048u;
+    g.cluster = c;
+    g.stage_bytes = stage;
+    g.stages = (int)(bound / stage);
+    if (g.stages > kSkinnyMaxStages) g.stages = kSkinnyMaxStages;
+    if (g.stages > kb) g.stages = kb;
+    if (g.stages < 1) g.stages = 1;
+    g.ring_bytes = (uint32_t)g.stages * stage;
+    if ((uint32_t)ncols * 512u > g.ring_bytes) g.ring_bytes = (uint32_t)ncols * 512u;
+    if (g.ring_bytes > bound || ncols > 512) return ATTT_ERR_INVALID_ARG;
+    g.tmem_cols = 32;
+    while ((int)g.tmem_cols < ncols) g.tmem_cols <<= 1;
+    if (!g.status) g.status = device_status_word(dev);
+    const size_t smem = 1024 + (size_t)g.ring_bytes + 8 * (2 * (size_t)g.stages + 1) + 16;
+    auto kern = tc_skinny_kernel<A_MN>;
+    if (!set_smem_limit(reinterpret_cast<const void *>(kern), smem, dev)) return ATTT_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(clusters * c));
+    cfg.blockDim = dim3(kSkinnyThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    unsigned na = 0;
+    if (pdl) {
+        attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[na].val.programmaticStreamSerializationAllowed = 1;
+        ++na;
+    }
+    if (c > 1) {
+        attr[na].id = cudaLaunchAttributeClusterDimension;
+        attr[na].val.clusterDim.x = (unsigned)c;
+        attr[na].val.clusterDim.y = 1;
+        attr[na].val.clusterDim.z = 1;
+        ++na;
+    }
+    cfg.attrs = attr;
+    cfg.numAttrs = na;
+    if (cudaLaunchKernelEx(&cfg, kern, maps, g) != cudaSuccess) return ATTT_ERR_CUDA;
+    count_launch();
+    return cudaGetLastError() == cudaSuccess ? ATTT_OK : ATTT_ERR_CUDA;
+}
+
+// A K-major A operand [rows, k] (128-row boxes) and an MN-major one [k, rows].
+static bool tmap_a(CUtensorMap *m, const void *p, int64_t k, int64_t rows) {
+    return make_tmap_bf16(m, p, (uint64_t)k, (uint64_t)rows, (uint64_t)k * 2, 64, 128);
+}
+static bool tmap_a_mn(CUtensorMap *m, const void *p, int64_t rows, int64_t k) {
+    return make_tmap_bf16(m, p, (uint64_t)rows, (uint64_t)k, (uint64_t)rows * 2, 64, 64);
+}
+
+// s16[m, c] = bf16(scale sum_k a[m, k] M[k, c]) for c < rpad (zero past r): M =
+// A [din, r] read MN-major (mn) or M^T = B [r, dout] read K-major.  `zero`:
+// counters of the next launch.
+// Whether s u or s v takes the skinny form, and on how many CTAs per tile (0:
+// the grouped form).  Fewer than kSkinnyMinBlocks K blocks leave a cluster
+// nothing to split.  Measured at 2,048 x 3,584, r 16: grouped 15 us (and 4 us of
+// prep for u), skinny 9.8; 403 rows 11 and 3.5 against 8.3.
+static int skinny_project_cluster(int64_t L, int64_t kb, int dev) {
+    return kb < kSkinnyMinBlocks ? 0 : skinny_cluster(cdiv(L, 128), kb, dev);
+}
+
+static attt_status skinny_project(const attt_bf16 *d_a, const attt_bf16 *d_m, int64_t L, int64_t K, int r, int rpad,
+                                  bool mn, float scale, __nv_bfloat16 *s16, unsigned int *zero, int nzero, int c,
+                                  int dev, cudaStream_t stream) {
+    SkinnyMaps maps;
+    SkinnyArgs g{};
+    if (!tmap_a(&maps.a[0], d_a, K, L)) return ATTT_ERR_INVALID_ARG;
+    const bool ok = mn ? make_tmap_bf16(&maps.b[0], d_m, (uint64_t)r, (uint64_t)K, (uint64_t)r * 2, 64, 64)
+                       : make_tmap_bf16(&maps.b[0], d_m, (uint64_t)K, (uint64_t)r, (uint64_t)K * 2, 64, (uint32_t)rpad);
+    if (!ok) return ATTT_ERR_INVALID_ARG;
+    g.ngroup = g.nmaps_a = g.nmaps_b = 1;
+    g.zero = zero;
+    g.nzero = nzero;
+    SkinnySeg &s = g.seg[0];
+    s.nb = 1; s.n = rpad; s.b_mn = mn ? 1 : 0; s.kb = (int)cdiv(K, 64); s.N = rpad;
+    s.out = GOUT_N16; s.alpha = scale; s.r = r; s.rpad = rpad; s.ld = rpad; s.out16 = s16;
+    g.grp[0] = SkinnyGroup{0, c, 0, 1, s.kb, (int)L, rpad};
+    return launch_skinny<false>(maps, g, cdiv(L, 128), c, false, dev, stream);
+}
+
+// How the passes of attt_lora_grad run as skinny launches: the clusters of each
+// pass; whether pass 1 gives u and every v_p of a row tile to one cluster
+// (merged) or to one each; and in pass 2, how many tiles of a dB_p share a
+// cluster (ratio) beside the wider dA tiles.  c1 = 0: the grouped stream-K form.
+struct SkinnyGradPlan {
+    int c1, c2, ratio;
+    bool merged;
+};
+
+static SkinnyGradPlan skinny_grad_plan(int64_t L, int64_t din, int nproj, const int64_t *dout, int r, int rpad,
+                                       int dev) {
+    SkinnyGradPlan p{0, 0, 1, true};
+    const int Nu = nproj * rpad;
+    if (r % 8 != 0 || nproj > kSkinnyMaxProj || Nu > kSkinnyMaxCols) return p;
+    const int64_t rows = cdiv(L, 128), ku = cdiv(din, 64), kl = cdiv(L, 64);
+    const double bu = skinny_block(nproj, rpad, true), bv = skinny_block(1, rpad, false);
+    int64_t kt = ku, kmin = ku, kmax = 0;
+    for (int q = 0; q < nproj; ++q) {
+        const int64_t k = cdiv(dout[q], 64);
+        kt += k;
+        if (k < kmin) kmin = k;
+        if (k > kmax) kmax = k;
+    }
+    if (kt < kSkinnyMinBlocks) return p;
+    double t1 = 1e30, t2 = 1e30;
+    const int cm = skinny_cluster(rows, kt, dev), cs = skinny_cluster(rows * (1 + nproj), kmin, dev);
+    if (cm > 0) {
+        t1 = cdiv(kt, cm) * (ku * bu + (kt - ku) * bv) / kt;
+        p.c1 = cm;
+    }
+    if (cs > 0) {
+        const double u = cdiv(ku, cs) * bu, v = cdiv(kmax, cs) * bv, t = u > v ? u : v;
+        if (t < t1) {
+            t1 = t;
+            p.c1 = cs;
+            p.merged = false;
+        }
+    }
+    const double ba = skinny_block(1, Nu, false);
+    for (int ratio = 1; ratio <= 2; ++ratio) {
+        int64_t n = cdiv(din, 128);
+        for (int q = 0; q < nproj; ++q) n += cdiv(cdiv(dout[q], 128), ratio);
+        int c = skinny_cluster(n, kl, dev);
+        c -= c % ratio;
+        if (c == 0) continue;
+        const double a = cdiv(kl, c) * ba, b = cdiv(kl, c / ratio) * bv, t = a > b ? a : b;
+        if (t < t2) {
+            t2 = t;
+            p.c2 = c;
+            p.ratio = ratio;
+        }
+    }
+    // The grouped form streams every block of both passes over all SMs, but pays
+    // for a prep launch and the ends of its tiles: the skinny form wins while its
+    // two passes stream for at most kSkinnyExtra microseconds longer (measured,
+    // grouped against skinny: L 2,048, q and v at r 16, +2.7: 27.0 -> 22.3 us; L
+    // 4,096, 14,336 -> 4,096 at r 32, +4.7: 63 -> 54; L 8,192, 4,096 -> 4,096 and
+    // 1,024 at r 8, +5.4: 58 -> 64; L 6,000, three projections at r 32, +12: 74 -> 85).
+    const int BN = Nu;  // every block of the grouped form carries this many B rows
+    int64_t t2n = cdiv(din, 128);
+    for (int q = 0; q < nproj; ++q) t2n += cdiv(dout[q], 128);
+    const double grouped = (double)(rows * kt + t2n * kl) * skinny_block(1, BN, false) / num_sms(dev);
+    if (p.c2 == 0 || t1 + t2 > grouped + kSkinnyExtra) p.c1 = 0;
+    return p;
+}
+
+// Both passes of attt_lora_grad as skinny launches (two launches, the adapters
+// read in place).  r is a multiple of 8 (rows of A are 16-byte multiples).
+static attt_status lora_grad_skinny(const attt_bf16 *d_x, int64_t L, int64_t din, int nproj,
+                                    const attt_bf16 *const *d_dy, const int64_t *dout, const attt_bf16 *const *d_A,
+                                    const attt_bf16 *const *d_B, int r, float scale, float *const *d_dA,
+                                    float *const *d_dB, const LoraLayout &c, const SkinnyGradPlan &pl, int *status,
+                                    int dev, cudaStream_t stream) {
+    {   // pass 1, 128 rows per tile: u^T = (x [A_0 | A_1 | ..])^T and every v_p^T = (dy_p B_p^T)^T
+        SkinnyMaps maps;
+        SkinnyArgs g{};
+        g.status = status;
+        if (!tmap_a(&maps.a[0], d_x, din, L)) return ATTT_ERR_INVALID_ARG;
+        SkinnySeg &u = g.seg[0];
+        u.nb = nproj; u.n = c.rpad; u.b_mn = 1; u.kb = (int)cdiv(din, 64); u.N = c.Nu;
+        u.out = GOUT_T16; u.alpha = 1.0f; u.out16 = c.uT16; u.ld = c.Lp; u.r = u.rpad = c.rpad;
+        int kb = u.kb;
+        for (int p = 0; p < nproj; ++p) {
+            if (!make_tmap_bf16(&maps.b[p], d_A[p], (uint64_t)r, (uint64_t)din, (uint64_t)r * 2, 64, 64) ||
+                !tmap_a(&maps.a[1 + p], d_dy[p], dout[p], L) ||
+                !make_tmap_bf16(&maps.b[nproj + p], d_B[p], (uint64_t)dout[p], (uint64_t)r, (uint64_t)dout[p] * 2, 64,
+                                (uint32_t)c.rpad))
+                return ATTT_ERR_INVALID_ARG;
+            SkinnySeg &v = g.seg[1 + p];
+            v.a = 1 + p; v.b = nproj + p; v.nb = 1; v.n = c.rpad; v.kb = (int)cdiv(dout[p], 64);
+            v.col = pl.merged ? c.Nu + p * c.rpad : 0; v.N = c.rpad;
+            v.out = GOUT_T16; v.alpha = 1.0f; v.out16 = c.vT16 + (size_t)p * c.rpad * c.Lp; v.ld = c.Lp;
+            v.r = v.rpad = c.rpad;
+            kb += v.kb;
+        }
+        g.nmaps_a = 1 + nproj; g.nmaps_b = 2 * nproj;
+        const int rows = (int)cdiv(L, 128);
+        if (pl.merged) {
+            g.ngroup = 1;
+            g.grp[0] = SkinnyGroup{0, pl.c1, 0, 1 + nproj, kb, (int)L, 2 * c.Nu};
+        } else {
+            g.ngroup = 1 + nproj;
+            for (int q = 0; q < g.ngroup; ++q)
+                g.grp[q] = SkinnyGroup{q * rows, pl.c1, q, 1, g.seg[q].kb, (int)L, q == 0 ? c.Nu : c.rpad};
+        }
+        const attt_status st = launch_skinny<false>(maps, g, (int64_t)rows * g.ngroup, pl.c1, false, dev, stream);
+        if (st != ATTT_OK) return st;
+    }
+    // pass 2, a tile per 128 columns of x (dA of every p) and of each dy_p (dB_p, stored transposed)
+    SkinnyMaps maps;
+    SkinnyArgs g{};
+    g.status = status;
+    const int kb = (int)cdiv(L, 64);
+    if (!tmap_a_mn(&maps.a[0], d_x, din, L) ||
+        !make_tmap_bf16(&maps.b[0], c.vT16, (uint64_t)L, (uint64_t)c.Nu, (uint64_t)c.Lp * 2, 64, (uint32_t)c.Nu) ||
+        !make_tmap_bf16(&maps.b[1], c.uT16, (uint64_t)L, (uint64_t)c.Nu, (uint64_t)c.Lp * 2, 64, (uint32_t)c.rpad))
+        return ATTT_ERR_INVALID_ARG;
+    SkinnySeg &a = g.seg[0];
+    a.nb = 1; a.n = c.Nu; a.kb = kb; a.N = c.Nu;
+    a.out = GOUT_N32; a.alpha = scale; a.r = r; a.rpad = c.rpad;
+    for (int p = 0; p < nproj; ++p) a.outp[p] = d_dA[p];
+    g.grp[0] = SkinnyGroup{0, pl.c2, 0, 1, kb, (int)din, c.Nu};
+    int64_t clusters = cdiv(din, 128);
+    for (int p = 0; p < nproj; ++p) {
+        if (!tmap_a_mn(&maps.a[1 + p], d_dy[p], dout[p], L)) return ATTT_ERR_INVALID_ARG;
+        SkinnySeg &b = g.seg[1 + p];
+        b.a = 1 + p; b.b = 1; b.nb = 1; b.n = c.rpad; b.b_n_off = p * c.rpad; b.kb = kb; b.N = c.rpad;
+        b.out = GOUT_T32; b.alpha = scale; b.out32 = d_dB[p]; b.ld = dout[p]; b.r = r; b.rpad = c.rpad;
+        g.grp[1 + p] = SkinnyGroup{(int)clusters, pl.c2 / pl.ratio, 1 + p, 1, kb, (int)dout[p], c.rpad};
+        clusters += cdiv(cdiv(dout[p], 128), pl.ratio);
+    }
+    g.ngroup = 1 + nproj; g.nmaps_a = 1 + nproj; g.nmaps_b = 2;
+    return launch_skinny<true>(maps, g, clusters, pl.c2, true, dev, stream);
+}
+
 attt_status lora_grad_run(const attt_bf16 *d_x, int64_t L, int64_t din, int nproj, const attt_bf16 *const *d_dy,
                           const int64_t *dout, const attt_bf16 *const *d_A, const attt_bf16 *const *d_B, int r,
                           float scale, float *const *d_dA, float *const *d_dB, void *d_ws, size_t ws_bytes,
@@ -353,6 +645,11 @@ attt_status lora_grad_run(const attt_bf16 *d_x, int64_t L, int64_t din, int npro
 
     LoraLayout c = lora_layout(d_ws, L, din, nproj, dout, r);
     const int BN = c.BN;
+    const SkinnyGradPlan pl = skinny_grad_plan(L, din, nproj, dout, r, c.rpad, dev);
+    if (pl.c1 > 0)
+        return lora_grad_skinny(d_x, L, din, nproj, d_dy, dout, d_A, d_B, r, scale, d_dA, d_dB, c, pl, status, dev,
+                                stream);
+
     // prep: adapters to K-major (rank padded with zeros), accumulators zeroed
     {
         PrepArgs a{};
@@ -788,6 +1085,11 @@ attt_status attt_lora_forward(const attt_bf16 *d_x, const attt_bf16 *d_W0, const
     st = current_device(&dev);
     if (st != ATTT_OK) return st;
     ProjLayout c = proj_layout(d_ws, L, din, dout, r, true);
+    const int cs = r % 8 == 0 ? skinny_project_cluster(L, cdiv(din, 64), dev) : 0;
+    if (cs > 0) {  // s u = s x A, A read in place
+        st = skinny_project(d_x, d_A, L, din, r, c.rpad, true, scale, c.s16, nullptr, 0, cs, dev, stream);
+        if (st != ATTT_OK) return st;
+    } else {
     {   // A^T (and B) padded to rpad rows, tickets zeroed
         PrepArgs a{};
         a.A[0] = reinterpret_cast<const __nv_bfloat16 *>(d_A);
@@ -810,6 +1112,7 @@ attt_status attt_lora_forward(const attt_bf16 *d_x, const attt_bf16 *d_W0, const
         u.out = GOUT_N16; u.out16 = c.s16; u.ld = c.rpad; u.alpha = scale; u.r = c.rpad; u.rpad = c.rpad;
         st = launch_group<false, false>(&u, 1, c.rpad, c.part, c.tickets, dev, stream, nullptr);
         if (st != ATTT_OK) return st;
+    }
     }
     {   // h = [x | s u] [W0 ; B]: W0 [din, dout] and B [r, dout] are read MN-major
         GemmProblem p{};
@@ -844,17 +1147,24 @@ attt_status attt_lora_input_grad(const attt_bf16 *d_dy, const attt_bf16 *d_W0, c
     st = current_device(&dev);
     if (st != ATTT_OK) return st;
     ProjLayout c = proj_layout(d_ws, L, din, dout, r, false);
-    if (cudaMemsetAsync(c.tickets, 0, sizeof(unsigned int) * (size_t)(c.tiles + kDxSplitRegions), stream) !=
-        cudaSuccess)
-        return ATTT_ERR_CUDA;
-    {   // s v = s dy B^T, bf16 [L, rpad]; B [r, dout] is the K-major operand (rows past r read as zeros)
-        GroupSpec v{};
-        v.a = d_dy; v.a_rows_ld = dout; v.a_rows = L; v.a_k = dout;
-        v.b = d_B; v.b_rows_ld = dout; v.b_rows = r; v.b_k = dout;
-        v.M = (int)L; v.N = c.rpad; v.K = (int)dout;
-        v.out = GOUT_N16; v.out16 = c.s16; v.ld = c.rpad; v.alpha = scale; v.r = c.rpad; v.rpad = c.rpad;
-        st = launch_group<false, false>(&v, 1, c.rpad, c.part, c.tickets, dev, stream, nullptr);
+    const int cs = skinny_project_cluster(L, cdiv(dout, 64), dev);
+    if (cs > 0) {  // s v = s dy B^T, and the tail split's counters zeroed
+        st = skinny_project(d_dy, d_B, L, dout, r, c.rpad, false, scale, c.s16, c.tickets + c.tiles, kDxSplitRegions,
+                            cs, dev, stream);
         if (st != ATTT_OK) return st;
+    } else {
+        if (cudaMemsetAsync(c.tickets, 0, sizeof(unsigned int) * (size_t)(c.tiles + kDxSplitRegions), stream) !=
+            cudaSuccess)
+            return ATTT_ERR_CUDA;
+        {   // s v = s dy B^T, bf16 [L, rpad]; B [r, dout] is the K-major operand (rows past r read as zeros)
+            GroupSpec v{};
+            v.a = d_dy; v.a_rows_ld = dout; v.a_rows = L; v.a_k = dout;
+            v.b = d_B; v.b_rows_ld = dout; v.b_rows = r; v.b_k = dout;
+            v.M = (int)L; v.N = c.rpad; v.K = (int)dout;
+            v.out = GOUT_N16; v.out16 = c.s16; v.ld = c.rpad; v.alpha = scale; v.r = c.rpad; v.rpad = c.rpad;
+            st = launch_group<false, false>(&v, 1, c.rpad, c.part, c.tickets, dev, stream, nullptr);
+            if (st != ATTT_OK) return st;
+        }
     }
     {   // dx = [dy | s v] [W0^T ; A^T]: W0 [din, dout] and A [din, r] are read K-major
         GemmProblem p{};

@@ -171,3 +171,24 @@ def test_ragged_shapes_and_repeatability(attt, L, din, douts, r):
     for p in range(len(douts)):
         assert np.array_equal(gA[p].view(np.uint32), hA[p].view(np.uint32)), ("dA", p)
         assert np.array_equal(gB[p].view(np.uint32), hB[p].view(np.uint32)), ("dB", p)
+
+
+@pytest.mark.parametrize("L,din,douts,r", [
+    (1, 1024, [1024], 16),                    # one row, one K block in pass 2
+    (93, 2056, [4104, 8], 8),                 # one tile per pass-1 problem; a dout of one vector
+    (411, 1032, [520, 264, 1000], 24),        # rank padded, ragged K blocks shared unevenly by a cluster
+    (1300, 640, [1288], 64),                  # 64 columns
+    (2100, 3584, [3584, 512], 16),            # u and v of a row tile on one cluster
+    (1000, 648, [2992, 1584, 3808, 1792], 32),  # two dB tiles share a cluster beside the wider dA tiles
+])
+def test_tiles_on_clusters(attt, L, din, douts, r):
+    """Groups whose tiles are few enough for clusters that split their K blocks
+    and sum through distributed shared memory: against the oracle, and two
+    calls give the same bits."""
+    host = _inputs(L + din + r, L, din, douts, r)
+    gA, gB = _check_group(attt, *host)
+    hA, hB = _group(attt, *host, 2.0)
+    for p in range(len(douts)):
+        assert np.array_equal(gA[p].view(np.uint32), hA[p].view(np.uint32)), ("dA", p)
+        assert np.array_equal(gB[p].view(np.uint32), hB[p].view(np.uint32)), ("dB", p)
+    assert attt.attt_device_status() == 0
