@@ -148,9 +148,14 @@ def _check(code: int, where: str) -> None:
         raise AtttError(code, where)
 
 
-def _stream(stream: Optional[torch.cuda.Stream]) -> ctypes.c_void_p:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+def _stream(stream: Optional[torch.cuda.Stream]) -> int:
+    """The cudaStream_t of `stream`, or of the current stream (asked for by its
+    handle: building a torch Stream object takes longer than a launch)."""
+    if stream is not None:
+        return stream.cuda_stream
+    if not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
@@ -170,12 +175,12 @@ def _bf16(t: torch.Tensor) -> int:
 
 
 def _expect(t: Optional[torch.Tensor], shape, dtype, name: str) -> None:
-    """Raises ValueError unless t (when given) has this shape and dtype: the
-    C ABI takes sizes on trust, so a smaller tensor would be read or written
-    past its end."""
+    """Raises ValueError unless t (when given) has this shape (a tuple of ints)
+    and dtype: the C ABI takes sizes on trust, so a smaller tensor would be read
+    or written past its end."""
     if t is None:
         return
-    if tuple(t.shape) != tuple(int(x) for x in shape):
+    if t.shape != shape:
         raise ValueError(f"{name}: expected shape {tuple(shape)}, got {tuple(t.shape)}")
     if t.dtype != dtype:
         raise ValueError(f"{name}: expected {dtype}, got {t.dtype}")
@@ -200,12 +205,12 @@ def attt_kernel_launches() -> int:
 
 def attt_selftest_wait_timeout(stream=None) -> None:
     """Launches the bounded-wait self-test (a wait that runs out after 2 s)."""
-    _check(load_library().attt_selftest_wait_timeout(_stream(stream)), "attt_selftest_wait_timeout")
+    _check((_lib or load_library()).attt_selftest_wait_timeout(_stream(stream)), "attt_selftest_wait_timeout")
 
 
 def attt_fault_inject(site: str) -> None:
     """One pending host-side fault: "alloc", "table_full" or "none"."""
-    _check(load_library().attt_fault_inject(site.encode()), "attt_fault_inject")
+    _check((_lib or load_library()).attt_fault_inject(site.encode()), "attt_fault_inject")
 
 
 def attt_device_status(stream=None) -> int:
@@ -266,13 +271,13 @@ def attt_history_destroy(h: History) -> None:
 
 
 def attt_history_reset(h: History, stream=None) -> None:
-    _check(load_library().attt_history_reset(h.handle, _stream(stream)), "attt_history_reset")
+    _check((_lib or load_library()).attt_history_reset(h.handle, _stream(stream)), "attt_history_reset")
 
 
 def attt_history_insert(h: History, tokens: torch.Tensor, stream=None) -> None:
     if tokens.dtype != torch.int32:
         raise ValueError("tokens must be int32")
-    _check(load_library().attt_history_insert(h.handle, _ptr(tokens), tokens.numel(), _stream(stream)),
+    _check((_lib or load_library()).attt_history_insert(h.handle, _ptr(tokens), tokens.numel(), _stream(stream)),
            "attt_history_insert")
 
 
@@ -311,7 +316,7 @@ def attt_history_count(h: History, ngrams: torch.Tensor, out: Optional[torch.Ten
     _expect(out, (m,), torch.int32, "out")
     if out is None:
         out = torch.empty(m, dtype=torch.int32, device=ngrams.device)
-    _check(load_library().attt_history_count(h.handle, _ptr(ngrams), m, _ptr(out), _stream(stream)),
+    _check((_lib or load_library()).attt_history_count(h.handle, _ptr(ngrams), m, _ptr(out), _stream(stream)),
            "attt_history_count")
     return out
 
@@ -325,8 +330,8 @@ def attt_ngram_weights(h: History, tokens: torch.Tensor, w_min: float = 0.05,
     _expect(out, (L,), torch.float32, "out")
     if out is None:
         out = torch.empty(L, dtype=torch.float32, device=tokens.device)
-    _check(load_library().attt_ngram_weights(h.handle, _ptr(tokens), L, float(w_min), _ptr(out), _stream(stream)),
-           "attt_ngram_weights")
+    _check((_lib or load_library()).attt_ngram_weights(
+        h.handle, _ptr(tokens), L, float(w_min), _ptr(out), _stream(stream)), "attt_ngram_weights")
     return out
 
 
@@ -366,7 +371,7 @@ def attt_weighted_ce_fwd_bwd(h: torch.Tensor, W: torch.Tensor, tgt: torch.Tensor
         workspace = torch.empty(attt_ce_workspace_bytes(L, d, V), dtype=torch.uint8, device=dev)
     if tgt.dtype != torch.int32 or w.dtype != torch.float32:
         raise ValueError("tgt must be int32 and w float32")
-    _check(load_library().attt_weighted_ce_fwd_bwd(
+    _check((_lib or load_library()).attt_weighted_ce_fwd_bwd(
         _bf16(h), _bf16(W), _ptr(tgt), _ptr(w), L, d, V, _ptr(loss), _ptr(dh), _ptr(lse),
         _ptr(workspace), workspace.numel(), _stream(stream)), "attt_weighted_ce_fwd_bwd")
     return loss, dh, lse
@@ -395,21 +400,43 @@ def _lora_check(x: torch.Tensor, dys, As, Bs, dAs, dBs):
         raise ValueError("at least one projection (dys) is required")
     if not (len(As) == len(Bs) == k) or (dAs is not None and len(dAs) != k) or (dBs is not None and len(dBs) != k):
         raise ValueError("dys, As, Bs (and dAs, dBs) must have one entry per projection")
-    _expect(x, (L, din), torch.bfloat16, "x")
+    bf16, f32 = torch.bfloat16, torch.float32
+    _expect(x, (L, din), bf16, "x")
     if As[0].dim() != 2:
         raise ValueError(f"As[0]: expected a 2-D [din, r] tensor, got shape {tuple(As[0].shape)}")
-    r = int(As[0].shape[1])
+    r = As[0].shape[1]
+    a_shape = (din, r)
     douts = []
     for p in range(k):
-        if dys[p].dim() != 2:
-            raise ValueError(f"dys[{p}]: expected a 2-D [L, dout] tensor, got shape {tuple(dys[p].shape)}")
-        douts.append(int(dys[p].shape[1]))
-        _expect(dys[p], (L, douts[p]), torch.bfloat16, f"dys[{p}]")
-        _expect(As[p], (din, r), torch.bfloat16, f"As[{p}]")
-        _expect(Bs[p], (r, douts[p]), torch.bfloat16, f"Bs[{p}]")
-        _expect(dAs[p] if dAs is not None else None, (din, r), torch.float32, f"dAs[{p}]")
-        _expect(dBs[p] if dBs is not None else None, (r, douts[p]), torch.float32, f"dBs[{p}]")
-    return int(L), int(din), r, douts
+        dy, A, B = dys[p], As[p], Bs[p]
+        if dy.dim() != 2:
+            raise ValueError(f"dys[{p}]: expected a 2-D [L, dout] tensor, got shape {tuple(dy.shape)}")
+        rows, dout = dy.shape
+        douts.append(dout)
+        # one test for the usual case; the named checks say what is wrong
+        if rows != L or dy.dtype != bf16 or A.shape != a_shape or A.dtype != bf16 or B.shape != (r, dout) \
+                or B.dtype != bf16:
+            _expect(dy, (L, dout), bf16, f"dys[{p}]")
+            _expect(A, a_shape, bf16, f"As[{p}]")
+            _expect(B, (r, dout), bf16, f"Bs[{p}]")
+        if dAs is not None and dAs[p] is not None and (dAs[p].shape != a_shape or dAs[p].dtype != f32):
+            _expect(dAs[p], a_shape, f32, f"dAs[{p}]")
+        if dBs is not None and dBs[p] is not None and (dBs[p].shape != (r, dout) or dBs[p].dtype != f32):
+            _expect(dBs[p], (r, dout), f32, f"dBs[{p}]")
+    return L, din, r, douts
+
+
+def _lora_arrays(dys, douts, As, Bs, dAs, dBs):
+    """The C call's six per-projection arrays as one buffer: (the buffer, which
+    must outlive the call, and the addresses of dy, dout, A, B, dA, dB)."""
+    k = len(dys)
+    vals = [_ptr(t) or 0 for t in dys]
+    vals += douts
+    for ts in (As, Bs, dAs, dBs):
+        vals += [_ptr(t) or 0 for t in ts]
+    buf = (ctypes.c_int64 * (6 * k))(*vals)
+    base = ctypes.addressof(buf)
+    return buf, [base + 8 * k * i for i in range(6)]
 
 
 def attt_lora_grad(x: torch.Tensor, dys: Sequence[torch.Tensor], As: Sequence[torch.Tensor],
@@ -426,12 +453,10 @@ def attt_lora_grad(x: torch.Tensor, dys: Sequence[torch.Tensor], As: Sequence[to
         dBs = [torch.empty(r, do, dtype=torch.float32, device=dev) for do in douts]
     if workspace is None:
         workspace = torch.empty(attt_lora_workspace_bytes(L, din, douts, r), dtype=torch.uint8, device=dev)
-    P = ctypes.c_void_p
-    arr = lambda ts, f: (P * k)(*[f(t) for t in ts])  # noqa: E731
-    douts_arr = (ctypes.c_int64 * k)(*douts)
-    _check(load_library().attt_lora_grad(
-        _bf16(x), L, din, k, arr(dys, _bf16), douts_arr, arr(As, _bf16), arr(Bs, _bf16), int(r), float(scale),
-        arr(dAs, _ptr), arr(dBs, _ptr), _ptr(workspace), workspace.numel(), _stream(stream)), "attt_lora_grad")
+    buf, (p_dy, p_dout, p_A, p_B, p_dA, p_dB) = _lora_arrays(dys, douts, As, Bs, dAs, dBs)
+    _check((_lib or load_library()).attt_lora_grad(
+        _bf16(x), L, din, k, p_dy, p_dout, p_A, p_B, r, float(scale), p_dA, p_dB, _ptr(workspace), workspace.numel(),
+        _stream(stream)), "attt_lora_grad")
     return dAs, dBs
 
 
@@ -449,12 +474,10 @@ def attt_lora_grad_noalloc(x: torch.Tensor, dys: Sequence[torch.Tensor], As: Seq
         raise ValueError("attt_lora_grad_noalloc: the caller passes the output tensors dAs and dBs")
     L, din, r, douts = _lora_check(x, dys, As, Bs, dAs, dBs)
     k = len(dys)
-    P = ctypes.c_void_p
-    arr = lambda ts, f: (P * k)(*[f(t) for t in ts])  # noqa: E731
-    douts_arr = (ctypes.c_int64 * k)(*douts)
-    _check(load_library().attt_lora_grad_noalloc(
-        _bf16(x), L, din, k, arr(dys, _bf16), douts_arr, arr(As, _bf16), arr(Bs, _bf16), int(r), float(scale),
-        arr(dAs, _ptr), arr(dBs, _ptr), _stream(stream)), "attt_lora_grad_noalloc")
+    buf, (p_dy, p_dout, p_A, p_B, p_dA, p_dB) = _lora_arrays(dys, douts, As, Bs, dAs, dBs)
+    _check((_lib or load_library()).attt_lora_grad_noalloc(
+        _bf16(x), L, din, k, p_dy, p_dout, p_A, p_B, r, float(scale), p_dA, p_dB, _stream(stream)),
+        "attt_lora_grad_noalloc")
     return dAs, dBs
 
 
@@ -469,7 +492,7 @@ def attt_lora_step(A32: torch.Tensor, B32: torch.Tensor, dA: torch.Tensor, dB: t
     _expect(dB, (r, dout), torch.float32, "dB")
     _expect(A16, (din, r), torch.bfloat16, "A16")
     _expect(B16, (r, dout), torch.bfloat16, "B16")
-    _check(load_library().attt_lora_step(
+    _check((_lib or load_library()).attt_lora_step(
         _ptr(A32), _ptr(B32), _ptr(dA), _ptr(dB), din, dout, r, float(lr),
         _bf16(A16) if A16 is not None else None, _bf16(B16) if B16 is not None else None, _stream(stream)),
         "attt_lora_step")
@@ -503,7 +526,7 @@ def attt_lora_forward(x: torch.Tensor, W0: torch.Tensor, A: torch.Tensor, B: tor
     if workspace is None:
         workspace = torch.empty(attt_lora_forward_workspace_bytes(L, din, dout, r), dtype=torch.uint8,
                                 device=x.device)
-    _check(load_library().attt_lora_forward(
+    _check((_lib or load_library()).attt_lora_forward(
         _bf16(x), _bf16(W0), _bf16(A), _bf16(B), L, din, dout, int(r), float(scale), _bf16(h), _ptr(workspace),
         workspace.numel(), _stream(stream)), "attt_lora_forward")
     return h
@@ -525,7 +548,7 @@ def attt_lora_input_grad(dy: torch.Tensor, W0: torch.Tensor, A: torch.Tensor, B:
     if workspace is None:
         workspace = torch.empty(attt_lora_input_grad_workspace_bytes(L, din, dout, r), dtype=torch.uint8,
                                 device=dy.device)
-    _check(load_library().attt_lora_input_grad(
+    _check((_lib or load_library()).attt_lora_input_grad(
         _bf16(dy), _bf16(W0), _bf16(A), _bf16(B), L, din, dout, int(r), float(scale), _ptr(dx), _ptr(workspace),
         workspace.numel(), _stream(stream)), "attt_lora_input_grad")
     return dx
@@ -539,7 +562,8 @@ def attt_cast_bf16(src: torch.Tensor, dst: Optional[torch.Tensor] = None, stream
         dst = torch.empty(src.shape, dtype=torch.bfloat16, device=src.device)
     if dst.numel() != src.numel():
         raise ValueError(f"dst: expected {src.numel()} elements, got {dst.numel()}")
-    _check(load_library().attt_cast_bf16(_ptr(src), _bf16(dst), src.numel(), _stream(stream)), "attt_cast_bf16")
+    _check((_lib or load_library()).attt_cast_bf16(_ptr(src), _bf16(dst), src.numel(), _stream(stream)),
+           "attt_cast_bf16")
     return dst
 
 
@@ -699,7 +723,7 @@ def attt_kl_drift(hp: torch.Tensor, hq: torch.Tensor, W: torch.Tensor, kl: Optio
         kl_mean = torch.empty(1, dtype=torch.float32, device=dev)
     if workspace is None:
         workspace = torch.empty(attt_kl_workspace_bytes(L, d, V), dtype=torch.uint8, device=dev)
-    _check(load_library().attt_kl_drift(_bf16(hp), _bf16(hq), _bf16(W), L, d, V, _ptr(kl), _ptr(kl_mean),
+    _check((_lib or load_library()).attt_kl_drift(_bf16(hp), _bf16(hq), _bf16(W), L, d, V, _ptr(kl), _ptr(kl_mean),
                                         _ptr(workspace), workspace.numel(), _stream(stream)), "attt_kl_drift")
     return kl, kl_mean
 
@@ -742,7 +766,7 @@ def attt_wordsets_destroy(s: WordSets) -> None:
 
 
 def attt_wordsets_reset(s: WordSets, stream=None) -> None:
-    _check(load_library().attt_wordsets_reset(s.handle, _stream(stream)), "attt_wordsets_reset")
+    _check((_lib or load_library()).attt_wordsets_reset(s.handle, _stream(stream)), "attt_wordsets_reset")
 
 
 def attt_wordsets_updates(s: WordSets) -> int:
@@ -768,7 +792,7 @@ def attt_repetition(s: WordSets, text: torch.Tensor, tau: float = 0.5, out: Opti
         keep = torch.empty(1, dtype=torch.int32, device=dev)
     n = text.numel()
     base = _ptr(out)
-    _check(load_library().attt_repetition(s.handle, _ptr(text) if n else None, n, float(tau), base, base + 4,
+    _check((_lib or load_library()).attt_repetition(s.handle, _ptr(text) if n else None, n, float(tau), base, base + 4,
                                           _ptr(keep), _stream(stream)), "attt_repetition")
     return out, keep
 
@@ -851,7 +875,7 @@ def attt_lora_adamw_step(A32: torch.Tensor, B32: torch.Tensor, dA: torch.Tensor,
     """In-place AdamW step on the fp32 masters (moments mA, vA, mB, vB), bf16 refresh."""
     din, r = A32.shape
     dout = B32.shape[1]
-    _check(load_library().attt_lora_adamw_step(
+    _check((_lib or load_library()).attt_lora_adamw_step(
         _ptr(A32), _ptr(B32), _ptr(dA), _ptr(dB), _ptr(mA), _ptr(vA), _ptr(mB), _ptr(vB), din, dout, r, float(lr),
         float(betas[0]), float(betas[1]), float(eps), float(weight_decay), int(step),
         _bf16(A16) if A16 is not None else None, _bf16(B16) if B16 is not None else None, _stream(stream)),
