@@ -21,7 +21,7 @@ namespace attt {
 
 constexpr int kKlBN = 256;  // 256-column tiles (the accumulator double-buffered: 512 TMEM columns)
 constexpr int kKlRows = 32;
-constexpr int kKlWarps = 8;
+constexpr int kKlWarps = 16;
 
 struct KlLayout {
     int64_t ntiles, plane, nblk;
@@ -44,8 +44,10 @@ static KlLayout kl_layout(void *ws, int64_t L, int64_t V) {
     return k;
 }
 
-// 32 rows per block (lane = row); warp w merges tiles t = w (mod 8) with
-// coalesced loads of the planes, then warp 0 merges the warps' results.
+// 32 rows per block (lane = row); warp w merges tiles t = w (mod 16) with
+// coalesced loads of the planes, four tiles' loads in flight (few rows leave
+// few blocks, and their latency bounds the kernel), then warp 0 merges the
+// warps' results.
 // Merge of (m, s, x) with (m2, s2, x2): M = max, s = s 2^(m-M) + s2 2^(m2-M),
 // x the same with x, x2.  The last block (ticket) sums the blocks' sums of
 // KL_j in block order for the mean.
@@ -59,19 +61,28 @@ __global__ void __launch_bounds__(kKlWarps * 32) kl_reduce_kernel(const float *_
     const int j = blockIdx.x * kKlRows + lane;
     float mp = -INFINITY, sp = 0.f, x = 0.f, mq = -INFINITY, sq = 0.f;
     if (j < L) {
-        for (int t = warp; t < ntiles; t += kKlWarps) {
-            const int64_t o = (int64_t)t * L + j;
-            const float m2 = __ldcg(part + o), s2 = __ldcg(part + plane + o);
-            const float n2 = __ldcg(part + 2 * plane + o), r2 = __ldcg(part + 3 * plane + o);
-            const float x2 = __ldcg(part + 4 * plane + o);
-            const float M = fmaxf(mp, m2);
-            const float a = exp2f(mp - M), b = exp2f(m2 - M);  // mp = -inf: a = 0
-            sp = sp * a + s2 * b;
-            x = x * a + x2 * b;
-            mp = M;
-            const float N = fmaxf(mq, n2);
-            sq = sq * exp2f(mq - N) + r2 * exp2f(n2 - N);
-            mq = N;
+        for (int t0 = warp; t0 < ntiles; t0 += 4 * kKlWarps) {
+            float v[4][5];  // four tiles' loads in flight together
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int t = t0 + k * kKlWarps;
+                const int64_t o = (int64_t)t * L + j;
+#pragma unroll
+                for (int i = 0; i < 5; ++i)
+                    v[k][i] = t < ntiles ? __ldcg(part + i * plane + o) : ((i == 0 || i == 2) ? -INFINITY : 0.f);
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (t0 + k * kKlWarps >= ntiles) break;
+                const float M = fmaxf(mp, v[k][0]);
+                const float a = exp2f(mp - M), b = exp2f(v[k][0] - M);  // mp = -inf: a = 0
+                sp = sp * a + v[k][1] * b;
+                x = x * a + v[k][4] * b;
+                mp = M;
+                const float N = fmaxf(mq, v[k][2]);
+                sq = sq * exp2f(mq - N) + v[k][3] * exp2f(v[k][2] - N);
+                mq = N;
+            }
         }
     }
     s_v[0][warp][lane] = mp;
