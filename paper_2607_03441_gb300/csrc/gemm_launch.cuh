@@ -30,6 +30,7 @@ struct GemmProblem {
     // operands_ready: A and B do not come from that grid.
     bool pdl = false;
     bool operands_ready = false;
+    bool second_waits = false;  // with operands_ready: A2 and B2 do come from it
     // Tail split (EPI_F32_ACC): workspace for up to `split_regions` partials
     // of 128 x BN fp32 and as many arrival counters (zero on entry).
     float *split_ws = nullptr;
@@ -270,7 +271,7 @@ attt_status launch_gemm(const GemmProblem &p, const EpiParams &ep, int dev, cuda
     g.b_n_off = p.b_n_off;
     g.b_k_off = p.b_k_off;
     g.tmem_cols = gemm_tmem_cols(p.BN);
-    g.operands_ready = p.operands_ready ? 1 : 0;
+    g.operands_ready = !p.operands_ready ? 0 : p.second_waits ? 2 : 1;
     g.status = status ? status : device_status_word(dev);
     g.ep = ep;
 

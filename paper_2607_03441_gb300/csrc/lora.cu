@@ -914,6 +914,7 @@ attt_status batch_forward(const attt_bf16 *d_x, const int64_t *off, int E, const
     p.b2 = c.BT; p.b2_rows_ld = d; p.b2_rows = d; p.b2_k = c.Ncat;
     p.M = (int)R; p.N = (int)d; p.K = (int)din; p.K2 = (int)c.Ncat;
     p.pdl = true;
+    p.operands_ready = p.second_waits = true;  // S follows the previous grid, the rest are inputs
     p.split_ws = c.split_ws; p.split_regions = kDxSplitRegions;
     EpiParams ep{};
     ep.out16 = reinterpret_cast<__nv_bfloat16 *>(d_h); ep.out_ld = d; ep.alpha = 1.0f;
@@ -1009,6 +1010,7 @@ attt_status batch_input_grad(const attt_bf16 *d_dy, const int64_t *off, int E, c
     p.b2 = c.ACAT; p.b2_rows_ld = c.Ncat; p.b2_rows = din; p.b2_k = c.Ncat;
     p.M = (int)R; p.N = (int)din; p.K = (int)d; p.K2 = (int)c.Ncat;
     p.pdl = true;
+    p.operands_ready = p.second_waits = true;  // S follows the previous grid, the rest are inputs
     p.split_ws = c.split_ws; p.split_tick = c.tickets + c.tiles; p.split_regions = kDxSplitRegions;
     EpiParams ep{};
     ep.out = d_dx; ep.out_ld = din; ep.accumulate = 0; ep.alpha = 1.0f;
@@ -1122,6 +1124,7 @@ attt_status attt_lora_forward(const attt_bf16 *d_x, const attt_bf16 *d_W0, const
         p.b2 = d_B; p.b2_rows_ld = dout; p.b2_rows = dout; p.b2_k = r;
         p.M = (int)L; p.N = (int)dout; p.K = (int)din; p.K2 = c.rpad;
         p.pdl = true;
+        p.operands_ready = p.second_waits = true;  // s16 follows the previous grid, the rest are inputs
         p.split_ws = c.split_ws; p.split_regions = kDxSplitRegions;
         EpiParams ep{};
         ep.out16 = reinterpret_cast<__nv_bfloat16 *>(d_h); ep.out_ld = dout; ep.alpha = 1.0f;
@@ -1174,6 +1177,7 @@ attt_status attt_lora_input_grad(const attt_bf16 *d_dy, const attt_bf16 *d_W0, c
         p.b2 = d_A; p.b2_rows_ld = r; p.b2_rows = din; p.b2_k = r;
         p.M = (int)L; p.N = (int)din; p.K = (int)dout; p.K2 = c.rpad;
         p.pdl = true;
+        p.operands_ready = p.second_waits = true;  // s16 follows the previous grid, the rest are inputs
         p.split_ws = c.split_ws; p.split_tick = c.tickets + c.tiles; p.split_regions = kDxSplitRegions;
         EpiParams ep{};
         ep.out = d_dx; ep.out_ld = din; ep.accumulate = 0; ep.alpha = 1.0f;

@@ -79,7 +79,8 @@ struct GemmArgs {
     uint32_t e_stage_bytes;  // shared-memory staging of the TMA-stored epilogue output, else 0
     // Programmatic dependent launch: the A/B operands were complete before the
     // previous grid in the stream started, so the producer need not wait for it
-    // (the epilogue always does).
+    // (the epilogue always does).  2: those of the first pair only; the producer
+    // waits before its first load of A2 / B2, which come last along K.
     int operands_ready;
     int kb_split;  // K blocks of the first operand pair; later ones come from A2 / B2
     int *status;
@@ -640,6 +641,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         if (elect_one()) {
             // ---------------- TMA producer ----------------
             if (!g.operands_ready) griddep_wait();
+            bool second_ready = g.operands_ready != 2;
             int stage = 0;
             uint32_t phase = 0;
             uint32_t issued_mask = 0, issued_parity = 0;  // per stage: last issue pending?
@@ -655,6 +657,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                     const uint32_t b_dst = smem_u32(sB + (size_t)stage * b_bytes);
                     // K block kb of the first pair, or K block kb - kb_split of the second
                     const bool sec = kb >= g.kb_split;
+                    if (sec && !second_ready) {
+                        griddep_wait();
+                        second_ready = true;
+                    }
                     const CUtensorMap *pa = sec ? &tmA2 : &tmA;
                     const CUtensorMap *pb = sec ? &tmB2 : &tmB;
                     const int ka = sec ? (kb - g.kb_split) * 64 : g.a_k_off + kb * 64;
@@ -877,6 +883,7 @@ __global__ void __launch_bounds__(kGemmPairThreads, 1)
         if (elect_one()) {
             // ---------------- TMA producers (both CTAs; warp 0 even, warp 6 odd stages) ----------------
             if (!g.operands_ready) griddep_wait();
+            bool second_ready = g.operands_ready != 2;
             const uint32_t pid = warp == 0 ? 0u : 1u;  // this producer's stages: pos % 2 == pid
             uint32_t pos = 0;
             int stage = 0;
@@ -904,6 +911,10 @@ __global__ void __launch_bounds__(kGemmPairThreads, 1)
                     const uint32_t b_dst = smem_u32(sB + (size_t)stage * b_bytes);
                     // K block kb of the first pair, or K block kb - kb_split of the second
                     const bool sec = kb >= g.kb_split;
+                    if (sec && !second_ready) {
+                        griddep_wait();
+                        second_ready = true;
+                    }
                     const CUtensorMap *pa = sec ? &tmA2 : &tmA;
                     const CUtensorMap *pb = sec ? &tmB2 : &tmB;
                     const int ka = sec ? (kb - g.kb_split) * 64 : g.a_k_off + kb * 64;
