@@ -83,6 +83,7 @@ struct GemmArgs {
     // waits before its first load of A2 / B2, which come last along K.
     int operands_ready;
     int kb_split;  // K blocks of the first operand pair; later ones come from A2 / B2
+    int group_m;   // row tiles per group of the tile order (0: all)
     int *status;
     EpiParams ep;
     // Tail split (tc_gemm_kernel / tc_gemm_pair_kernel): tiles [0, whole_tiles)
@@ -158,6 +159,13 @@ __device__ __forceinline__ Work work_item(const GemmArgs &g, int w, int tiles_m)
         t = g.whole_tiles + k.tail;
         k.kb0 = (int)((int64_t)g.kb_total * k.piece / g.tail_s);
         k.kb1 = (int)((int64_t)g.kb_total * (k.piece + 1) / g.tail_s);
+    }
+    if (g.group_m > 0) {  // groups of group_m row tiles, m fastest within a group
+        const int per = g.group_m * g.tiles_n, gr = t / per, r = t - gr * per;
+        const int rows = min(g.group_m, tiles_m - gr * g.group_m);
+        k.tn = r / rows;
+        k.tm = gr * g.group_m + r - k.tn * rows;
+        return k;
     }
     k.tn = t / tiles_m;
     k.tm = t - k.tn * tiles_m;
