@@ -58,6 +58,10 @@ attt_status ngram_weights_batch(attt_history *const *hs, int E, const int32_t *d
 attt_status history_insert_batch(attt_history *const *hs, int E, const int32_t *d_tokens, const int64_t *off,
                                  cudaStream_t stream);
 
+// Zeroes a (and b, when not nullptr): 16-byte aligned, sizes multiples of 16
+// (ngram.cu).
+attt_status clear_tables(void *a, size_t a_bytes, void *b, size_t b_bytes, cudaStream_t stream);
+
 // Eq. 10 as attt_weighted_ce_fwd_bwd, with per-row normalisers `row_scale`
 // (dh_j = w_j row_scale_j (...); nullptr: 1/L for every row) and the per-row
 // NLL lse_j - z_{j,t_j} into `nll` (nullptr: not written) (ce.cu).

@@ -208,6 +208,49 @@ __device__ __forceinline__ void insert_block(const HistTokens &ht, int64_t p_beg
     }
 }
 
+// Zeroes up to two ranges of 16-byte words (tables of a reset), four stores in
+// flight per thread.  A reset's tables are next touched by the append's atomics
+// in L2, where these stores leave them.
+__global__ void __launch_bounds__(256) clear_kernel(uint4 *a, int64_t na, uint4 *b, int64_t nb) {
+    griddep_launch_dependents();
+    griddep_wait();
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x, t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll 4
+    for (int64_t i = t; i < na; i += stride) a[i] = z;
+#pragma unroll 4
+    for (int64_t i = t; i < nb; i += stride) b[i] = z;
+}
+
+// A launch of `kern` as a programmatic dependent of the previous kernel of the
+// stream: its blocks may be resident when that kernel ends.  Every kernel
+// launched so waits (griddep_wait) before it reads or writes global memory.
+template <class... P, class... A>
+static attt_status launch_dependent(void (*kern)(P...), dim3 grid, unsigned threads, cudaStream_t stream, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, kern, P(args)...) != cudaSuccess) return ATTT_ERR_CUDA;
+    count_launch();
+    return cudaGetLastError() == cudaSuccess ? ATTT_OK : ATTT_ERR_CUDA;
+}
+
+attt_status clear_tables(void *a, size_t a_bytes, void *b, size_t b_bytes, cudaStream_t stream) {
+    const int64_t na = (int64_t)(a_bytes / 16), nb = (int64_t)(b_bytes / 16);
+    int dev;
+    const attt_status st = current_device(&dev);
+    if (st != ATTT_OK) return st;
+    const int64_t want = cdiv(na > nb ? na : nb, 256 * 4), most = (int64_t)num_sms(dev) * 8;
+    return launch_dependent(clear_kernel, dim3((unsigned)(want < 1 ? 1 : want < most ? want : most)), 256, stream,
+                            static_cast<uint4 *>(a), na, static_cast<uint4 *>(b), nb);
+}
+
 // src (may be null): the appended tokens, new_len - old_len of them, not yet
 // in the stream; the launch copies them to hist[old_len, new_len) besides
 // inserting (one D2D copy fewer per append).
@@ -215,6 +258,8 @@ __global__ void __launch_bounds__(256) history_insert_kernel(int32_t *hist, cons
                                                              int64_t old_len, int64_t new_len, int64_t p_begin,
                                                              int64_t count, int n, Slot *table,
                                                              unsigned long long mask, int *status) {
+    griddep_launch_dependents();
+    griddep_wait();
     if (src) {
         const int64_t stride = (int64_t)gridDim.x * blockDim.x;
         for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < new_len - old_len; j += stride)
@@ -303,6 +348,8 @@ __global__ void __launch_bounds__(kWThreads) ngram_weights_kernel(const int32_t 
                                                                const int32_t *__restrict__ hist, int64_t hist_len,
                                                                const Slot *table, unsigned long long mask,
                                                                float w_min, float *__restrict__ w) {
+    griddep_launch_dependents();
+    griddep_wait();
     weights_block(x, L, n, hist, hist_len, table, mask, w_min, w, nullptr, 0.0f, (int64_t)blockIdx.x * kWTile);
 }
 
@@ -404,8 +451,8 @@ attt_status attt_history_destroy(attt_history *h) {
 attt_status attt_history_reset(attt_history *h, attt_stream stream) {
     ATTT_NVTX_RANGE();
     if (!h) return ATTT_ERR_INVALID_ARG;
-    if (cudaMemsetAsync(h->d_table, 0, h->capacity * sizeof(attt::Slot), stream) != cudaSuccess)
-        return ATTT_ERR_CUDA;
+    const attt_status st = attt::clear_tables(h->d_table, h->capacity * sizeof(attt::Slot), nullptr, 0, stream);
+    if (st != ATTT_OK) return st;
     h->len = 0;
     return ATTT_OK;
 }
@@ -443,13 +490,10 @@ attt_status attt_history_insert(attt_history *h, const int32_t *d_tokens, int64_
                    ? ATTT_OK
                    : ATTT_ERR_CUDA;
     }
-    const int threads = 256;
     const int64_t blocks = (count + attt::kInsTile - 1) / attt::kInsTile;
-    attt::history_insert_kernel<<<(unsigned)blocks, threads, 0, stream>>>(h->d_tokens, d_tokens, old_len, new_len,
-                                                                          p_begin, count, h->n, h->d_table,
-                                                                          h->capacity - 1, h->d_status);
-    attt::count_launch();
-    return cudaGetLastError() == cudaSuccess ? ATTT_OK : ATTT_ERR_CUDA;
+    return attt::launch_dependent(attt::history_insert_kernel, dim3((unsigned)blocks), 256, stream, h->d_tokens,
+                                  d_tokens, old_len, new_len, p_begin, count, h->n, h->d_table, h->capacity - 1,
+                                  h->d_status);
 }
 
 attt_status attt_history_save(const attt_history *h, int32_t *host_tokens, attt_stream stream) {
@@ -589,10 +633,8 @@ attt_status attt_ngram_weights(const attt_history *h, const int32_t *d_tokens, i
         return ATTT_ERR_INVALID_ARG;
     if (L == 0) return ATTT_OK;
     const int64_t blocks = (L + attt::kWTile - 1) / attt::kWTile;
-    attt::ngram_weights_kernel<<<(unsigned)blocks, attt::kWThreads, 0, stream>>>(
-        d_tokens, L, h->n, h->d_tokens, h->len, h->d_table, h->capacity - 1, w_min, d_w);
-    attt::count_launch();
-    return cudaGetLastError() == cudaSuccess ? ATTT_OK : ATTT_ERR_CUDA;
+    return attt::launch_dependent(attt::ngram_weights_kernel, dim3((unsigned)blocks), attt::kWThreads, stream,
+                                  d_tokens, L, h->n, h->d_tokens, h->len, h->d_table, h->capacity - 1, w_min, d_w);
 }
 
 }  // extern "C"

@@ -377,9 +377,9 @@ attt_status attt_wordsets_destroy(attt_wordsets *s) {
 attt_status attt_wordsets_reset(attt_wordsets *s, attt_stream stream) {
     ATTT_NVTX_RANGE();
     if (!s) return ATTT_ERR_INVALID_ARG;
-    if (cudaMemsetAsync(s->d_keys, 0, s->capacity * sizeof(unsigned long long), stream) != cudaSuccess ||
-        cudaMemsetAsync(s->d_masks, 0, s->capacity * s->W * sizeof(unsigned long long), stream) != cudaSuccess)
-        return ATTT_ERR_CUDA;
+    const attt_status st = attt::clear_tables(s->d_keys, s->capacity * sizeof(unsigned long long), s->d_masks,
+                                              s->capacity * s->W * sizeof(unsigned long long), stream);
+    if (st != ATTT_OK) return st;
     s->len = 0;
     s->count = 0;
     return ATTT_OK;
