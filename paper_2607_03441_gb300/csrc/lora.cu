@@ -231,9 +231,9 @@ struct GroupSpec {
     float *outp[kMaxProj];
 };
 
-// Limits of the skinny form (tc_skinny.cuh): ring slots, projections (a slot
-// holds a 64-column box per adapter) and columns.
-constexpr int kSkinnyMaxStages = 12, kSkinnyMaxProj = 4, kSkinnyMaxCols = 192;
+// Limits of the skinny form (tc_skinny.cuh): projections (a slot holds a
+// 64-column box per adapter) and columns.
+constexpr int kSkinnyMaxProj = 4, kSkinnyMaxCols = 192;
 constexpr int kSkinnyMinBlocks = 8;
 constexpr double kSkinnyExtra = 5.0;  // microseconds (skinny_grad_plan)
 constexpr int kGroupMinStages = 2;
@@ -389,6 +389,36 @@ static int skinny_cluster(int64_t tiles, int64_t kb, int dev) {
     return c;
 }
 
+// Fills in group gr's K ranges for `split` CTAs per tile: equal cost where every
+// CTA then has a block, else equal counts (at least one block each: split is at
+// most the blocks).
+static void skinny_split(const SkinnyArgs &g, SkinnyGroup &gr) {
+    int kt = 0;
+    double total = 0.0, cost[kSkinnySegs];
+    for (int i = 0; i < gr.nseg; ++i) {
+        const SkinnySeg &s = g.seg[gr.seg0 + i];
+        cost[i] = skinny_block(s.nb, s.n, s.b_mn != 0);
+        kt += s.kb;
+        total += s.kb * cost[i];
+    }
+    gr.kb[0] = 0;
+    gr.kb[gr.split] = kt;
+    int i = 0, at = 0;      // segment, and its first block
+    double before = 0.0;    // cost of the segments before it
+    for (int c = 1; c < gr.split; ++c) {
+        if (kt < 4 * gr.split) {
+            gr.kb[c] = kt * c / gr.split;
+            continue;
+        }
+        const double want = total * c / gr.split;
+        while (before + g.seg[gr.seg0 + i].kb * cost[i] < want) {
+            before += g.seg[gr.seg0 + i].kb * cost[i];
+            at += g.seg[gr.seg0 + i++].kb;
+        }
+        gr.kb[c] = at + (int)((want - before) / cost[i] + 0.5);
+    }
+}
+
 // Launches the groups of g (its groups, segments, tiles and columns filled in)
 // on `clusters` clusters of `c` CTAs.  `pdl`: a programmatic dependent of the
 // previous kernel.  False in *fits (nothing launched) if the accumulators of a
@@ -396,32 +426,31 @@ static int skinny_cluster(int64_t tiles, int64_t kb, int dev) {
 template <bool A_MN>
 static attt_status launch_skinny(const SkinnyMaps &maps, SkinnyArgs &g, int64_t clusters, int c, bool pdl, int dev,
                                  cudaStream_t stream) {
-    uint32_t stage = 0;
-    int ncols = 0, kb = 0;  // columns and K blocks of one CTA at most
+    uint32_t ring = 0;  // the most a CTA can use: a slot per K block, up to kSkinnyMaxStages
+    int ncols = 0;
     for (int q = 0; q < g.ngroup; ++q) {
-        const SkinnyGroup &gr = g.grp[q];
+        SkinnyGroup &gr = g.grp[q];
+        skinny_split(g, gr);
         if (gr.ncols > ncols) ncols = gr.ncols;
-        if (cdiv(gr.kb_total, gr.split) > kb) kb = (int)cdiv(gr.kb_total, gr.split);
+        int kb = 0;
+        for (int i = 0; i < gr.split; ++i)
+            if (gr.kb[i + 1] - gr.kb[i] > kb) kb = gr.kb[i + 1] - gr.kb[i];
+        if (kb > kSkinnyMaxStages) kb = kSkinnyMaxStages;
         for (int i = gr.seg0; i < gr.seg0 + gr.nseg; ++i) {
             const SkinnySeg &s = g.seg[i];
             const uint32_t b = kABytes + (uint32_t)s.nb * (s.b_mn ? 8192u : (uint32_t)s.n * 128u);
-            if (b > stage) stage = b;
+            if ((uint32_t)kb * b > ring) ring = (uint32_t)kb * b;
         }
     }
-    const uint32_t bound = (uint32_t)kMaxSmem - 2048u;
+    const uint32_t bound = ((uint32_t)kMaxSmem - 2048u) / 1024u * 1024u;
     g.cluster = c;
-    g.stage_bytes = stage;
-    g.stages = (int)(bound / stage);
-    if (g.stages > kSkinnyMaxStages) g.stages = kSkinnyMaxStages;
-    if (g.stages > kb) g.stages = kb;
-    if (g.stages < 1) g.stages = 1;
-    g.ring_bytes = (uint32_t)g.stages * stage;
+    g.ring_bytes = ring < bound ? ring : bound;
     if ((uint32_t)ncols * 512u > g.ring_bytes) g.ring_bytes = (uint32_t)ncols * 512u;
     if (g.ring_bytes > bound || ncols > 512) return ATTT_ERR_INVALID_ARG;
     g.tmem_cols = 32;
     while ((int)g.tmem_cols < ncols) g.tmem_cols <<= 1;
     if (!g.status) g.status = device_status_word(dev);
-    const size_t smem = 1024 + (size_t)g.ring_bytes + 8 * (2 * (size_t)g.stages + 1) + 16;
+    const size_t smem = 1024 + (size_t)g.ring_bytes + 8 * (2 * kSkinnyMaxStages + 1) + 16;
     auto kern = tc_skinny_kernel<A_MN>;
     if (!set_smem_limit(reinterpret_cast<const void *>(kern), smem, dev)) return ATTT_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
@@ -484,7 +513,7 @@ static attt_status skinny_project(const attt_bf16 *d_a, const attt_bf16 *d_m, in
     SkinnySeg &s = g.seg[0];
     s.nb = 1; s.n = rpad; s.b_mn = mn ? 1 : 0; s.kb = (int)cdiv(K, 64); s.N = rpad;
     s.out = GOUT_N16; s.alpha = scale; s.r = r; s.rpad = rpad; s.ld = rpad; s.out16 = s16;
-    g.grp[0] = SkinnyGroup{0, c, 0, 1, s.kb, (int)L, rpad};
+    g.grp[0] = SkinnyGroup{0, c, 0, 1, (int)L, rpad, {}};
     return launch_skinny<false>(maps, g, cdiv(L, 128), c, false, dev, stream);
 }
 
@@ -569,7 +598,6 @@ static attt_status lora_grad_skinny(const attt_bf16 *d_x, int64_t L, int64_t din
         SkinnySeg &u = g.seg[0];
         u.nb = nproj; u.n = c.rpad; u.b_mn = 1; u.kb = (int)cdiv(din, 64); u.N = c.Nu;
         u.out = GOUT_T16; u.alpha = 1.0f; u.out16 = c.uT16; u.ld = c.Lp; u.r = u.rpad = c.rpad;
-        int kb = u.kb;
         for (int p = 0; p < nproj; ++p) {
             if (!make_tmap_bf16(&maps.b[p], d_A[p], (uint64_t)r, (uint64_t)din, (uint64_t)r * 2, 64, 64) ||
                 !tmap_a(&maps.a[1 + p], d_dy[p], dout[p], L) ||
@@ -581,17 +609,16 @@ static attt_status lora_grad_skinny(const attt_bf16 *d_x, int64_t L, int64_t din
             v.col = pl.merged ? c.Nu + p * c.rpad : 0; v.N = c.rpad;
             v.out = GOUT_T16; v.alpha = 1.0f; v.out16 = c.vT16 + (size_t)p * c.rpad * c.Lp; v.ld = c.Lp;
             v.r = v.rpad = c.rpad;
-            kb += v.kb;
         }
         g.nmaps_a = 1 + nproj; g.nmaps_b = 2 * nproj;
         const int rows = (int)cdiv(L, 128);
         if (pl.merged) {
             g.ngroup = 1;
-            g.grp[0] = SkinnyGroup{0, pl.c1, 0, 1 + nproj, kb, (int)L, 2 * c.Nu};
+            g.grp[0] = SkinnyGroup{0, pl.c1, 0, 1 + nproj, (int)L, 2 * c.Nu, {}};
         } else {
             g.ngroup = 1 + nproj;
             for (int q = 0; q < g.ngroup; ++q)
-                g.grp[q] = SkinnyGroup{q * rows, pl.c1, q, 1, g.seg[q].kb, (int)L, q == 0 ? c.Nu : c.rpad};
+                g.grp[q] = SkinnyGroup{q * rows, pl.c1, q, 1, (int)L, q == 0 ? c.Nu : c.rpad, {}};
         }
         const attt_status st = launch_skinny<false>(maps, g, (int64_t)rows * g.ngroup, pl.c1, false, dev, stream);
         if (st != ATTT_OK) return st;
@@ -609,14 +636,14 @@ static attt_status lora_grad_skinny(const attt_bf16 *d_x, int64_t L, int64_t din
     a.nb = 1; a.n = c.Nu; a.kb = kb; a.N = c.Nu;
     a.out = GOUT_N32; a.alpha = scale; a.r = r; a.rpad = c.rpad;
     for (int p = 0; p < nproj; ++p) a.outp[p] = d_dA[p];
-    g.grp[0] = SkinnyGroup{0, pl.c2, 0, 1, kb, (int)din, c.Nu};
+    g.grp[0] = SkinnyGroup{0, pl.c2, 0, 1, (int)din, c.Nu, {}};
     int64_t clusters = cdiv(din, 128);
     for (int p = 0; p < nproj; ++p) {
         if (!tmap_a_mn(&maps.a[1 + p], d_dy[p], dout[p], L)) return ATTT_ERR_INVALID_ARG;
         SkinnySeg &b = g.seg[1 + p];
         b.a = 1 + p; b.b = 1; b.nb = 1; b.n = c.rpad; b.b_n_off = p * c.rpad; b.kb = kb; b.N = c.rpad;
         b.out = GOUT_T32; b.alpha = scale; b.out32 = d_dB[p]; b.ld = dout[p]; b.r = r; b.rpad = c.rpad;
-        g.grp[1 + p] = SkinnyGroup{(int)clusters, pl.c2 / pl.ratio, 1 + p, 1, kb, (int)dout[p], c.rpad};
+        g.grp[1 + p] = SkinnyGroup{(int)clusters, pl.c2 / pl.ratio, 1 + p, 1, (int)dout[p], c.rpad, {}};
         clusters += cdiv(cdiv(dout[p], 128), pl.ratio);
     }
     g.ngroup = 1 + nproj; g.nmaps_a = 1 + nproj; g.nmaps_b = 2;

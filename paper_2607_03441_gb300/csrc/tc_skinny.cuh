@@ -21,7 +21,8 @@
 // A tile is a list of segments laid end to end along K, each with its own A
 // and B operands and its own accumulator columns: the u and every v_p of a row
 // tile in the first pass, one segment in the others.  The i-th of the c CTAs
-// that share a tile takes the K blocks [i KT / c, (i + 1) KT / c) of the list.
+// that share a tile takes the K blocks [kb[i], kb[i + 1]) of the list, about the
+// same cost each (skinny_split).
 #pragma once
 
 #include "tc_gemm.cuh"
@@ -32,6 +33,7 @@ namespace attt {
 constexpr int kSkinnyThreads = 192;  // producer, MMA, four epilogue warps
 constexpr int kSkinnySegs = kMaxProj + 1;
 constexpr int kSkinnyMaxCluster = 8;
+constexpr int kSkinnyMaxStages = 12;  // ring slots (barriers) of a CTA
 
 struct SkinnySeg {
     int a, b;     // tensor maps: the A operand, the first of nb B operands
@@ -54,7 +56,8 @@ struct SkinnySeg {
 // clusters from cluster_begin; `split` CTAs share a tile (a cluster of C holds
 // C / split tiles).
 struct SkinnyGroup {
-    int cluster_begin, split, seg0, nseg, kb_total, M, ncols;
+    int cluster_begin, split, seg0, nseg, M, ncols;
+    int kb[kSkinnyMaxCluster + 1];  // first K block of each of the `split` CTAs, then the total
 };
 
 struct SkinnyMaps {
@@ -63,8 +66,8 @@ struct SkinnyMaps {
 };
 
 struct SkinnyArgs {
-    int ngroup, nmaps_a, nmaps_b, cluster, stages;
-    uint32_t stage_bytes, ring_bytes, tmem_cols;
+    int ngroup, nmaps_a, nmaps_b, cluster;
+    uint32_t ring_bytes, tmem_cols;
     int *status;
     unsigned int *zero;  // words set to zero (a later launch's counters), or nullptr
     int nzero;
@@ -81,31 +84,39 @@ __device__ __forceinline__ float4 ld_cluster_f4(uint32_t addr) {
     return v;
 }
 
-// Columns [n, n + 4) of row m of a segment's result.
-__device__ __forceinline__ void skinny_store(const SkinnySeg &s, int m, int n, const float4 &f) {
-    const float v[4] = {s.alpha * f.x, s.alpha * f.y, s.alpha * f.z, s.alpha * f.w};
-    if (s.out == GOUT_T16) {
+// Sums the column quads [qd, qe) of this thread's row over the nc <= J CTAs
+// whose partials start (at this row) at cb[0..nc), in that order, and hands
+// each to store(column, sum): U J loads in flight, no division and no look into
+// the kernel's parameters per quad (with those, one quad took 0.45 us and the
+// 48 of a 192-column tile 22 us of a 69 us pass).
+template <int U, int J, class Store>
+__device__ __forceinline__ void skinny_sum(int qd, int qe, int nc, const uint32_t (&cb)[kSkinnyMaxCluster],
+                                           Store &&store) {
+    for (; qd < qe; qd += U) {
+        float4 f[U][J];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-            if (n + i < s.N) s.out16[(int64_t)(n + i) * s.ld + m] = __float2bfloat16_rn(v[i]);
-    } else if (s.out == GOUT_N32) {
-        const int blk = n / s.rpad, c = n - blk * s.rpad;
-        float *o = s.outp[blk] + (int64_t)m * s.r + c;
-        if (c + 4 <= s.r && (reinterpret_cast<uintptr_t>(o) & 15) == 0) {
-            *reinterpret_cast<float4 *>(o) = make_float4(v[0], v[1], v[2], v[3]);
-        } else {
+        for (int u = 0; u < U; ++u)
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-                if (c + i < s.r) o[i] = v[i];
+            for (int j = 0; j < J; ++j)
+                f[u][j] = j < nc && qd + u < qe ? ld_cluster_f4(cb[j] + (uint32_t)(qd + u) * 2048u)
+                                                : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            float4 t = f[u][0];
+#pragma unroll
+            for (int j = 1; j < J; ++j)
+                if (j < nc) { t.x += f[u][j].x; t.y += f[u][j].y; t.z += f[u][j].z; t.w += f[u][j].w; }
+            if (qd + u < qe) store(4 * (qd + u), t);
         }
-    } else if (s.out == GOUT_T32) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-            if (n + i < s.r) s.out32[(int64_t)(n + i) * s.ld + m] = v[i];
-    } else {  // GOUT_N16: ld a multiple of 16, the base 256-byte aligned
-        __nv_bfloat162 b[2] = {__floats2bfloat162_rn(v[0], v[1]), __floats2bfloat162_rn(v[2], v[3])};
-        *reinterpret_cast<uint2 *>(s.out16 + (int64_t)m * s.ld + n) = *reinterpret_cast<uint2 *>(b);
     }
+}
+
+template <class Store>
+__device__ __forceinline__ void skinny_sum_any(int qd, int qe, int nc, const uint32_t (&cb)[kSkinnyMaxCluster],
+                                               Store &&store) {
+    if (nc <= 2) skinny_sum<8, 2>(qd, qe, nc, cb, store);
+    else if (nc <= 4) skinny_sum<4, 4>(qd, qe, nc, cb, store);
+    else skinny_sum<2, 8>(qd, qe, nc, cb, store);
 }
 
 template <bool A_MN>
@@ -113,13 +124,32 @@ __global__ void __launch_bounds__(kSkinnyThreads, 1)
     tc_skinny_kernel(const __grid_constant__ SkinnyMaps maps, const __grid_constant__ SkinnyArgs g) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    const int S = g.stages;
     const uint32_t ring = smem_u32(smem);  // later the CTA's partial accumulators
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + g.ring_bytes);
-    const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + S), done = smem_u32(bars + 2 * S);
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * S + 1);
+    const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + kSkinnyMaxStages),
+                   done = smem_u32(bars + 2 * kSkinnyMaxStages);
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * kSkinnyMaxStages + 1);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+    const int rank = g.cluster > 1 ? (int)cluster_ctarank() : 0;
+    const int cid = blockIdx.x / g.cluster;
+    int q = 0;
+    while (q + 1 < g.ngroup && cid >= g.grp[q + 1].cluster_begin) ++q;
+    const SkinnyGroup &gr = g.grp[q];
+    const int C = gr.split, first = rank - rank % C, part = rank % C;  // the CTAs that share this tile
+    const int m0 = ((cid - gr.cluster_begin) * (g.cluster / C) + first / C) * 128;
+    const int seg0 = gr.seg0, seg1 = gr.seg0 + gr.nseg;
+    const int k0 = gr.kb[part], k1 = m0 < gr.M ? gr.kb[part + 1] : k0;
+    // the ring: slots of the largest block this CTA loads, as many as fit (blocks
+    // from HBM take 1.5 us and more: five slots hold a CTA to 0.3 us a block)
+    uint32_t stage_bytes = kABytes;
+    for (int si = seg0, base = 0; si < seg1; base += g.seg[si++].kb) {
+        const SkinnySeg &s = g.seg[si];
+        if (max(k0, base) < min(k1, base + s.kb))
+            stage_bytes = max(stage_bytes, kABytes + (uint32_t)s.nb * (s.b_mn ? 8192u : (uint32_t)s.n * 128u));
+    }
+    const int S = min(kSkinnyMaxStages, (int)(g.ring_bytes / stage_bytes));
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
@@ -144,16 +174,6 @@ __global__ void __launch_bounds__(kSkinnyThreads, 1)
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
 
-    const int rank = g.cluster > 1 ? (int)cluster_ctarank() : 0;
-    const int cid = blockIdx.x / g.cluster;
-    int q = 0;
-    while (q + 1 < g.ngroup && cid >= g.grp[q + 1].cluster_begin) ++q;
-    const SkinnyGroup &gr = g.grp[q];
-    const int C = gr.split, first = rank - rank % C, part = rank % C;  // the CTAs that share this tile
-    const int m0 = ((cid - gr.cluster_begin) * (g.cluster / C) + first / C) * 128;
-    const int kt = gr.kb_total, seg0 = gr.seg0, seg1 = gr.seg0 + gr.nseg;
-    const int k0 = kt * part / C, k1 = m0 < gr.M ? kt * (part + 1) / C : k0;
-
     if (warp == 0) {
         if (elect_one()) {
             griddep_wait();  // the operands may come from the previous grid
@@ -173,7 +193,7 @@ __global__ void __launch_bounds__(kSkinnyThreads, 1)
                         ok = false;
                         break;
                     }
-                    const uint32_t a_dst = ring + (uint32_t)slot * g.stage_bytes;
+                    const uint32_t a_dst = ring + (uint32_t)slot * stage_bytes;
                     mbar_arrive_expect_tx(fb, bytes);
                     if (!A_MN) {
                         tma_load_2d(a_dst, ta, fb, k * 64, m0);
@@ -227,7 +247,7 @@ __global__ void __launch_bounds__(kSkinnyThreads, 1)
                     const int next = slot + 1 == S ? 0 : slot + 1;
                     const uint32_t next_phase = next == 0 ? phase ^ 1u : phase;
                     ready = mbar_test_wait(full0 + 8 * next, next_phase);
-                    const uint32_t a_addr = ring + (uint32_t)slot * g.stage_bytes;
+                    const uint32_t a_addr = ring + (uint32_t)slot * stage_bytes;
                     const uint64_t ad = smem_desc_sw128(a_addr, A_MN ? 8192 : 16, 1024);
                     for (int i = 0; i < nb; ++i) {
                         const uint64_t bd = smem_desc_sw128(a_addr + kABytes + 8192u * i, b_mn ? 8192 : 16, 1024);
@@ -292,31 +312,75 @@ __global__ void __launch_bounds__(kSkinnyThreads, 1)
     }
     if (warp >= 2 && m0 < gr.M) {
         const int m = m0 + row;
-        const int nq = gr.ncols / 4;
-        int si = seg0, base = 0, c0 = 0, c1 = 0, at = -1;
-        for (int qd = nq * part / C; qd < nq * (part + 1) / C; ++qd) {
-            while (4 * qd >= g.seg[si].col + g.seg[si].nb * g.seg[si].n) base += g.seg[si++].kb;
+        const int nq = gr.ncols / 4, q1 = nq * (part + 1) / C;
+        int base = 0;
+        for (int si = seg0; si < seg1; base += g.seg[si++].kb) {
             const SkinnySeg &s = g.seg[si];
-            if (at != si) {  // the CTAs that hold K blocks of this segment
-                at = si;
-                c0 = C;
-                for (int j = 0; j < C; ++j)
-                    if (max(kt * j / C, base) < min(kt * (j + 1) / C, base + s.kb)) {
-                        if (c0 == C) c0 = j;
-                        c1 = j;
-                    }
+            // the quads of columns of this segment in this CTA's share, and the CTAs
+            // [c0, c0 + nc) that hold K blocks of it
+            int qd = max(nq * part / C, s.col / 4);
+            const int qe = min(q1, (s.col + s.nb * s.n) / 4);
+            if (qd >= qe) continue;
+            int c0 = 0, nc = 0;
+            for (int j = 0; j < C; ++j)
+                if (max(gr.kb[j], base) < min(gr.kb[j + 1], base + s.kb)) {
+                    if (nc == 0) c0 = j;
+                    ++nc;
+                }
+            uint32_t cb[kSkinnyMaxCluster];
+#pragma unroll
+            for (int j = 0; j < kSkinnyMaxCluster; ++j)
+                cb[j] = mapa_shared(ring + (uint32_t)row * 16u, (uint32_t)(first + min(c0 + j, C - 1)));
+            // the sums' columns are the tile's; the segment's start at col.  Rows past
+            // the problem are summed (the loads are harmless) and not stored.
+            const int col = s.col, N = s.N, r = s.r;
+            const bool live = m < gr.M;
+            const float al = s.alpha;
+            const int64_t ld = s.ld;
+            if (s.out == GOUT_T16) {
+                __nv_bfloat16 *o = s.out16 + m - (int64_t)col * ld;
+                skinny_sum_any(qd, qe, nc, cb, [&](int n, const float4 &t) {
+                    const float v[4] = {al * t.x, al * t.y, al * t.z, al * t.w};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (live && n + i - col < N) o[(int64_t)(n + i) * ld] = __float2bfloat16_rn(v[i]);
+                });
+            } else if (s.out == GOUT_N32) {
+                // projection by projection: a block of rpad columns each
+                const int rpad = s.rpad;
+                for (int blk = (4 * qd - col) / rpad; qd < qe; ++blk) {
+                    const int be = min(qe, (col + (blk + 1) * rpad) / 4), c0b = col + blk * rpad;
+                    float *o = s.outp[blk] + (int64_t)m * r;
+                    const bool vec = (r & 3) == 0 && (reinterpret_cast<uintptr_t>(s.outp[blk]) & 15) == 0;
+                    skinny_sum_any(qd, be, nc, cb, [&](int n, const float4 &t) {
+                        const float v[4] = {al * t.x, al * t.y, al * t.z, al * t.w};
+                        const int c = n - c0b;
+                        if (live && vec && c + 4 <= r) {
+                            *reinterpret_cast<float4 *>(o + c) = make_float4(v[0], v[1], v[2], v[3]);
+                        } else {
+#pragma unroll
+                            for (int i = 0; i < 4; ++i)
+                                if (live && c + i < r) o[c + i] = v[i];
+                        }
+                    });
+                    qd = be;
+                }
+            } else if (s.out == GOUT_T32) {
+                float *o = s.out32 + m - (int64_t)col * ld;
+                skinny_sum_any(qd, qe, nc, cb, [&](int n, const float4 &t) {
+                    const float v[4] = {al * t.x, al * t.y, al * t.z, al * t.w};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (live && n + i - col < r) o[(int64_t)(n + i) * ld] = v[i];
+                });
+            } else {  // GOUT_N16: ld a multiple of 16, the base 256-byte aligned
+                __nv_bfloat16 *o = s.out16 + (int64_t)m * ld - col;
+                skinny_sum_any(qd, qe, nc, cb, [&](int n, const float4 &t) {
+                    __nv_bfloat162 b[2] = {__floats2bfloat162_rn(al * t.x, al * t.y),
+                                           __floats2bfloat162_rn(al * t.z, al * t.w)};
+                    if (live) *reinterpret_cast<uint2 *>(o + n) = *reinterpret_cast<uint2 *>(b);
+                });
             }
-            const uint32_t addr = ring + (uint32_t)(qd * 128 + row) * 16u;
-            float4 f[kSkinnyMaxCluster];
-#pragma unroll
-            for (int j = 0; j < kSkinnyMaxCluster; ++j)  // the loads in flight together
-                if (c0 + j <= c1)
-                    f[j] = C > 1 ? ld_cluster_f4(mapa_shared(addr, (uint32_t)(first + c0 + j))) : ld_shared_f4(addr);
-            float4 t = f[0];
-#pragma unroll
-            for (int j = 1; j < kSkinnyMaxCluster; ++j)
-                if (c0 + j <= c1) { t.x += f[j].x; t.y += f[j].y; t.z += f[j].z; t.w += f[j].w; }
-            if (m < gr.M) skinny_store(s, m, 4 * qd - s.col, t);
         }
     }
     if (g.cluster > 1) cluster_sync();  // no CTA leaves while another reads its partials
