@@ -60,6 +60,16 @@ __device__ __forceinline__ void griddep_launch_dependents() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// Takes the next number of a device-wide ticket: releases what this thread
+// wrote before it, and what a barrier ordered before it from the threads of its
+// block, to the block that takes the last number, which acquires all of it; one
+// atomic instead of two fences around a relaxed one.
+__device__ __forceinline__ unsigned int ticket_acq_rel(unsigned int *ticket) {
+    unsigned int n;
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(n) : "l"(ticket) : "memory");
+    return n;
+}
+
 // bar.sync on a named barrier shared by `count` threads (a multiple of 32).
 __device__ __forceinline__ void named_barrier_sync(uint32_t id, uint32_t count) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");

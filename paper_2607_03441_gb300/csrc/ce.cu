@@ -27,8 +27,8 @@ namespace attt {
 constexpr int kCeBN = 256;
 constexpr int kCeMinBN = 64;      // the narrowest tile of the logits contraction
 constexpr int kCeMaxTiles = 1024;  // chunk width at most, in kCeBN columns
-constexpr int kChunkWarps = 16;  // ce_chunk_kernel: 16 warps, 32 rows (one per lane) per block
-constexpr int kChunkRows = 32;
+constexpr int kChunkWarps = 16;  // ce_chunk_kernel: 16 warps of 4 tiles x 8 rows
+constexpr int kChunkRows = 8;    // rows per block: lane & 7
 // fp32 partials of 128 x kCeBN (128 KB each) for the K pieces of the dh
 // contraction (40 MB): two pieces for every SM of a 160-SM part.
 constexpr int kCeSplitRegions = 320;
@@ -174,10 +174,11 @@ struct CeChunkArgs {
     int *status;
 };
 
-// Bookkeeping of one chunk, 32 rows per block (lane = row), log2 units:
-//   warp k reads the chunk's tiles t = k (mod 16) with coalesced loads of
-//   part[t, rows], four in flight (one chunk may hold 600 tiles and few rows:
-//   the loads' latency bounds the kernel); per row the chunk max M_c and the
+// Bookkeeping of one chunk, 8 rows per block, log2 units:
+//   64 lane groups each read every 64th of the chunk's tiles, 64 bytes of
+//   part[t, rows] per tile, four tiles in flight (one chunk may hold 600 tiles
+//   and few rows: the loads' latency bounds the kernel; at 93 rows and 594
+//   tiles 32 rows per block took 12.7 us); per row the chunk max M_c and the
 //   chunk's (max, sum) pair, merged into the running pair (lm, ls);
 //   R = mref, the reference GEMM1 wrote this chunk's E against.  A tile whose
 //   max exceeded R by more than kCeRefJump used its own max, and then
@@ -198,16 +199,29 @@ __global__ void __launch_bounds__(kChunkWarps * 32) ce_chunk_kernel(const CeChun
     griddep_wait();  // the chunk's logits contraction has completed
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int j0 = blockIdx.x * kChunkRows;
-    const int j = j0 + lane;
+    const int rl = lane & (kChunkRows - 1), sub = lane / kChunkRows;  // row of the block, tile of the warp's four
+    const int j = j0 + rl;
     const int L = a.L;
+    constexpr int kStreams = kChunkWarps * 32 / kChunkRows;
+    // the row's own terms, on their way while the tiles are merged
+    float mref0 = 0.f, w0 = 0.f, zt0 = 0.f;
+    int t0 = 0;
+    if (warp == 0 && sub == 0 && j < L) {
+        mref0 = a.mref[j];
+        if (a.last) {
+            t0 = a.tgt[j];
+            w0 = a.w[j];
+            zt0 = __ldcg(a.ztgt + j);
+        }
+    }
     float m = -INFINITY, s = 0.f;
     if (j < L) {
-        for (int t = warp; t < a.ntiles; t += 4 * kChunkWarps) {
+        for (int t = warp * (32 / kChunkRows) + sub; t < a.ntiles; t += 4 * kStreams) {
             float2 p[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                p[k] = t + k * kChunkWarps < a.ntiles ? __ldcg(a.part + (int64_t)(t + k * kChunkWarps) * L + j)
-                                                      : make_float2(-INFINITY, 0.f);
+                p[k] = t + k * kStreams < a.ntiles ? __ldcg(a.part + (int64_t)(t + k * kStreams) * L + j)
+                                                   : make_float2(-INFINITY, 0.f);
             const float mx = fmaxf(m, fmaxf(fmaxf(p[0].x, p[1].x), fmaxf(p[2].x, p[3].x)));
             if (mx == -INFINITY) continue;
             s *= exp2f(m - mx);
@@ -216,15 +230,23 @@ __global__ void __launch_bounds__(kChunkWarps * 32) ce_chunk_kernel(const CeChun
             m = mx;
         }
     }
-    s_m[warp][lane] = m;
-    s_s[warp][lane] = s;
+    for (int o = kChunkRows; o < 32; o <<= 1)
+        lse_merge(m, s, __shfl_xor_sync(0xffffffffu, m, o), __shfl_xor_sync(0xffffffffu, s, o));
+    if (sub == 0) {
+        s_m[warp][rl] = m;
+        s_s[warp][rl] = s;
+    }
     __syncthreads();
     if (warp == 0) {
-        for (int k = 1; k < kChunkWarps; ++k) lse_merge(m, s, s_m[k][lane], s_s[k][lane]);
-        const float mc = m;  // the chunk's max
+        m = -INFINITY;
+        s = 0.f;
+        for (int k = sub; k < kChunkWarps; k += 32 / kChunkRows) lse_merge(m, s, s_m[k][rl], s_s[k][rl]);
+        for (int o = kChunkRows; o < 32; o <<= 1)
+            lse_merge(m, s, __shfl_xor_sync(0xffffffffu, m, o), __shfl_xor_sync(0xffffffffu, s, o));
+        const float mc = m;  // the chunk's max; the row's terms are formed by the first lane of each row
         int rw = 0;
         float r = 0.f, contrib = 0.f;
-        if (j < L) {
+        if (j < L && sub == 0) {
             if (!a.first) {  // running pair first, then this chunk's
                 float rm = a.lm[j], rs = a.ls[j];
                 lse_merge(rm, rs, m, s);
@@ -233,7 +255,7 @@ __global__ void __launch_bounds__(kChunkWarps * 32) ce_chunk_kernel(const CeChun
             }
             a.lm[j] = m;
             a.ls[j] = s;
-            r = a.mref[j];
+            r = mref0;
             rw = (mc - r > kCeRefJump) ? 1 : 0;
             const float rp = rw ? mc : r;
             const float aold = a.first ? -INFINITY : a.aref[j];
@@ -246,18 +268,18 @@ __global__ void __launch_bounds__(kChunkWarps * 32) ce_chunk_kernel(const CeChun
                 const float lse2 = m + log2f(s);
                 const float lse = lse2 * 0.69314718055994531f;
                 if (a.lse_out) a.lse_out[j] = lse;
-                const int t = a.tgt[j];
-                const float c = a.w[j] * (a.row_scale ? a.row_scale[j] : a.inv_L);
+                const int t = t0;
+                const float c = w0 * (a.row_scale ? a.row_scale[j] : a.inv_L);
                 float nll;
                 if (t < 0 || t >= a.V) {
                     record_error(a.status, ATTT_ERR_TOKEN_RANGE);
                     nll = __int_as_float(0x7fc00000);
                     a.gamma[j] = __int_as_float(0x7fc00000);
                 } else {
-                    nll = lse - __ldcg(a.ztgt + j);
+                    nll = lse - zt0;
                     a.gamma[j] = c;
                 }
-                contrib = a.w[j] * nll;
+                contrib = w0 * nll;
                 if (a.nll_out) a.nll_out[j] = nll;
                 const float f = c * exp2f(anew - lse2);
                 al *= f;
@@ -266,15 +288,16 @@ __global__ void __launch_bounds__(kChunkWarps * 32) ce_chunk_kernel(const CeChun
             a.alpha[j] = al;
             a.beta[j] = be;
         }
-        s_rw[lane] = rw;
-        s_r[lane] = r;
-        s_mcf[lane] = mc;
+        if (sub == 0) {
+            s_rw[rl] = rw;
+            s_r[rl] = r;
+            s_mcf[rl] = mc;
+        }
         if (a.last) {
             for (int o = 16; o > 0; o >>= 1) contrib += __shfl_xor_sync(0xffffffffu, contrib, o);
             if (lane == 0) {
                 a.block_sums[blockIdx.x] = contrib;
-                __threadfence();
-                s_last = atomicAdd(a.ticket, 1u) == gridDim.x - 1;
+                s_last = ticket_acq_rel(a.ticket) == gridDim.x - 1;
             }
         }
     }
@@ -304,7 +327,6 @@ __global__ void __launch_bounds__(kChunkWarps * 32) ce_chunk_kernel(const CeChun
         }
     }
     if (a.last && s_last && warp == 0) {  // a fixed order: lane sums of blocks lane (mod 32), then a tree
-        __threadfence();
         float total = 0.f;
         for (unsigned i = lane; i < gridDim.x; i += 32) total += __ldcg(a.block_sums + i);
         for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);

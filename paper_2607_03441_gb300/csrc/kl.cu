@@ -20,7 +20,7 @@
 namespace attt {
 
 constexpr int kKlBN = 256;  // 256-column tiles (the accumulator double-buffered: 512 TMEM columns)
-constexpr int kKlRows = 32;
+constexpr int kKlRows = 8;  // rows per reduction block: lane & 7
 constexpr int kKlWarps = 16;
 
 struct KlLayout {
@@ -44,91 +44,92 @@ static KlLayout kl_layout(void *ws, int64_t L, int64_t V) {
     return k;
 }
 
-// 32 rows per block (lane = row); warp w merges tiles t = w (mod 16) with
-// coalesced loads of the planes, four tiles' loads in flight (few rows leave
-// few blocks, and their latency bounds the kernel), then warp 0 merges the
-// warps' results.
-// Merge of (m, s, x) with (m2, s2, x2): M = max, s = s 2^(m-M) + s2 2^(m2-M),
-// x the same with x, x2.  The last block (ticket) sums the blocks' sums of
-// KL_j in block order for the mean.
+// One row's five numbers over some of its tiles.  merge: M = max(m, m2), s = s
+// 2^(m-M) + s2 2^(m2-M), x the same with x, x2; a part without tiles (m2 =
+// -inf) adds nothing.
+struct KlPart {
+    float mp, sp, x, mq, sq;
+    __device__ __forceinline__ void merge(const KlPart &o) {
+        if (o.mp != -INFINITY) {
+            const float M = fmaxf(mp, o.mp), a = exp2f(mp - M), b = exp2f(o.mp - M);  // mp = -inf: a = 0
+            sp = sp * a + o.sp * b;
+            x = x * a + o.x * b;
+            mp = M;
+        }
+        if (o.mq != -INFINITY) {
+            const float N = fmaxf(mq, o.mq);
+            sq = sq * exp2f(mq - N) + o.sq * exp2f(o.mq - N);
+            mq = N;
+        }
+    }
+    __device__ __forceinline__ KlPart shfl_xor(int o) const {
+        return KlPart{__shfl_xor_sync(0xffffffffu, mp, o), __shfl_xor_sync(0xffffffffu, sp, o),
+                      __shfl_xor_sync(0xffffffffu, x, o), __shfl_xor_sync(0xffffffffu, mq, o),
+                      __shfl_xor_sync(0xffffffffu, sq, o)};
+    }
+};
+
+// 8 rows per block (lane & 7); 64 lane groups merge every 64th tile, four
+// tiles' loads in flight (few rows leave few blocks, and their latency bounds
+// the kernel: at 403 rows and 594 tiles, 32 rows per block and one tile per
+// round trip took 63 us), then the groups' results merge through shuffles and
+// shared memory in a fixed order.  The last block (ticket) sums the blocks'
+// sums of KL_j for the mean, in a fixed order too.
 __global__ void __launch_bounds__(kKlWarps * 32) kl_reduce_kernel(const float *__restrict__ part, int64_t plane,
                                                                  int ntiles, int L, float *kl_rows, float *kl_mean,
                                                                  float *block_sums, unsigned int *ticket) {
-    __shared__ float s_v[5][kKlWarps][kKlRows];
+    __shared__ KlPart s_v[kKlWarps][kKlRows];
     __shared__ bool s_last;
     griddep_wait();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int j = blockIdx.x * kKlRows + lane;
-    float mp = -INFINITY, sp = 0.f, x = 0.f, mq = -INFINITY, sq = 0.f;
+    const int rl = lane & (kKlRows - 1), sub = lane / kKlRows;
+    const int j = blockIdx.x * kKlRows + rl;
+    constexpr int kStreams = kKlWarps * 32 / kKlRows;
+    KlPart acc{-INFINITY, 0.f, 0.f, -INFINITY, 0.f};
     if (j < L) {
-        for (int t0 = warp; t0 < ntiles; t0 += 4 * kKlWarps) {
-            float v[4][5];  // four tiles' loads in flight together
+        for (int t0 = warp * (32 / kKlRows) + sub; t0 < ntiles; t0 += 4 * kStreams) {
+            KlPart v[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const int t = t0 + k * kKlWarps;
+                const int t = t0 + k * kStreams;
                 const int64_t o = (int64_t)t * L + j;
-#pragma unroll
-                for (int i = 0; i < 5; ++i)
-                    v[k][i] = t < ntiles ? __ldcg(part + i * plane + o) : ((i == 0 || i == 2) ? -INFINITY : 0.f);
+                v[k] = t < ntiles ? KlPart{__ldcg(part + o), __ldcg(part + plane + o), __ldcg(part + 4 * plane + o),
+                                           __ldcg(part + 2 * plane + o), __ldcg(part + 3 * plane + o)}
+                                  : KlPart{-INFINITY, 0.f, 0.f, -INFINITY, 0.f};
             }
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                if (t0 + k * kKlWarps >= ntiles) break;
-                const float M = fmaxf(mp, v[k][0]);
-                const float a = exp2f(mp - M), b = exp2f(v[k][0] - M);  // mp = -inf: a = 0
-                sp = sp * a + v[k][1] * b;
-                x = x * a + v[k][4] * b;
-                mp = M;
-                const float N = fmaxf(mq, v[k][2]);
-                sq = sq * exp2f(mq - N) + v[k][3] * exp2f(v[k][2] - N);
-                mq = N;
-            }
+            for (int k = 0; k < 4; ++k) acc.merge(v[k]);
         }
     }
-    s_v[0][warp][lane] = mp;
-    s_v[1][warp][lane] = sp;
-    s_v[2][warp][lane] = x;
-    s_v[3][warp][lane] = mq;
-    s_v[4][warp][lane] = sq;
+    for (int o = kKlRows; o < 32; o <<= 1) acc.merge(acc.shfl_xor(o));
+    if (sub == 0) s_v[warp][rl] = acc;
     __syncthreads();
     if (warp == 0) {
+        acc = KlPart{-INFINITY, 0.f, 0.f, -INFINITY, 0.f};
+        for (int w = sub; w < kKlWarps; w += 32 / kKlRows) acc.merge(s_v[w][rl]);
+        for (int o = kKlRows; o < 32; o <<= 1) acc.merge(acc.shfl_xor(o));
         float kl = 0.f;
-        if (j < L) {
-            for (int w = 1; w < kKlWarps; ++w) {
-                const float m2 = s_v[0][w][lane], s2 = s_v[1][w][lane], x2 = s_v[2][w][lane];
-                const float n2 = s_v[3][w][lane], r2 = s_v[4][w][lane];
-                if (m2 != -INFINITY) {
-                    const float M = fmaxf(mp, m2);
-                    const float a = exp2f(mp - M), b = exp2f(m2 - M);
-                    sp = sp * a + s2 * b;
-                    x = x * a + x2 * b;
-                    mp = M;
-                }
-                if (n2 != -INFINITY) {
-                    const float N = fmaxf(mq, n2);
-                    sq = sq * exp2f(mq - N) + r2 * exp2f(n2 - N);
-                    mq = N;
-                }
-            }
-            const float dl = ((mp + log2f(sp)) - (mq + log2f(sq))) * 0.69314718055994531f;
-            kl = x / sp - dl;
+        if (j < L && sub == 0) {
+            const float dl = ((acc.mp + log2f(acc.sp)) - (acc.mq + log2f(acc.sq))) * 0.69314718055994531f;
+            kl = acc.x / acc.sp - dl;
             if (kl_rows) kl_rows[j] = kl;
         }
         float sum = kl;
         for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
         if (lane == 0) {
             block_sums[blockIdx.x] = sum;
-            __threadfence();
-            s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+            s_last = ticket_acq_rel(ticket) == gridDim.x - 1;
         }
     }
     __syncthreads();
-    if (s_last && threadIdx.x == 0) {
-        __threadfence();
+    if (s_last && warp == 0) {
         float total = 0.f;
-        for (unsigned b = 0; b < gridDim.x; ++b) total += __ldcg(block_sums + b);
-        if (kl_mean) *kl_mean = total / (float)L;
-        *ticket = 0u;
+        for (unsigned b = lane; b < gridDim.x; b += 32) total += __ldcg(block_sums + b);
+        for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
+        if (lane == 0) {
+            if (kl_mean) *kl_mean = total / (float)L;
+            *ticket = 0u;
+        }
     }
 }
 

@@ -274,9 +274,7 @@ __global__ void __launch_bounds__(kInsThreads) repetition_kernel(RepArgs a) {
     if (threadIdx.x == 0 && s_distinct) atomicAdd(a.distinct, s_distinct);
     __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();  // the block's counts (ordered before by the barrier) precede its ticket
-        s_last = atomicAdd(a.ticket, 1u) == gridDim.x - 1;
-        __threadfence();
+        s_last = attt::ticket_acq_rel(a.ticket) == gridDim.x - 1;
     }
     __syncthreads();
     if (!s_last) return;
