@@ -25,7 +25,7 @@
 namespace attt {
 
 constexpr int kCeBN = 256;
-constexpr int kCeMinBN = 64;      // the narrowest tile of the logits contraction
+constexpr int kCeMinSet = 32;     // columns of the narrowest set (half a 64-column tile) of the logits contraction
 constexpr int kCeMaxTiles = 1024;  // chunk width at most, in kCeBN columns
 constexpr int kChunkWarps = 16;  // ce_chunk_kernel: 16 warps of 4 tiles x 8 rows
 constexpr int kChunkRows = 8;    // rows per block: lane & 7
@@ -88,7 +88,7 @@ static CeLayout ce_layout(void *ws, int64_t L, int64_t d, int64_t V) {
     c.Vc = ce_chunk_max(L, V);
     c.nblk = cdiv(L, kChunkRows);
     Carve cv{static_cast<char *>(ws), 0};
-    c.part = cv.take<float2>((size_t)(cdiv(c.Vc, kCeMinBN) * L));
+    c.part = cv.take<float2>((size_t)(cdiv(c.Vc, kCeMinSet) * L));
     c.ztgt = cv.take<float>((size_t)L);
     c.block_sums = cv.take<float>((size_t)c.nblk);
     c.aref = cv.take<float>((size_t)L);
@@ -154,8 +154,8 @@ __global__ void __launch_bounds__(256) ce_ref_kernel(const __nv_bfloat16 *__rest
 }
 
 struct CeChunkArgs {
-    const float2 *part;  // [vocab tiles of the chunk, L] (max, sum) of every tile (log2 units)
-    int ntiles, tile_w, L, V;  // tile_w: columns per tile
+    const float2 *part;  // [sets of tile_w columns of the chunk, L] (max, sum) of each (log2 units)
+    int ntiles, tile_w, L, V;
     __nv_bfloat16 *G;
     int64_t G_ld;
     float *aref, *mref, *lm, *ls, *alpha, *beta, *gamma;
@@ -416,7 +416,9 @@ attt_status ce_fwd_bwd_run(const attt_bf16 *d_h, const attt_bf16 *d_W, const int
     const CePlan plan = ce_plan(L, d, V, c.split_regions, num_sms(dev));
     for (int64_t v0 = 0, ci = 0; v0 < V; v0 += plan.Vc, ++ci) {
         const int64_t Nc = (V - v0 < plan.Vc) ? V - v0 : plan.Vc;
-        const int ntiles = (int)cdiv(Nc, plan.logits.BN);
+        const int sets = cdiv(d, 64) <= kTwoSetBlocks ? 2 : 1;
+        const int width = plan.logits.BN / sets;  // columns of a tile that one epilogue set takes
+        const int ntiles = (int)cdiv(Nc, width);
         const bool last = v0 + Nc >= V;
         {   // GEMM1: logits of the chunk -> per-tile stats and E = exp(z - R)
             GemmProblem p{};
@@ -430,11 +432,12 @@ attt_status ce_fwd_bwd_run(const attt_bf16 *d_h, const attt_bf16 *d_W, const int
             ep.tgt = d_tgt; ep.part = c.part; ep.tile0 = 0; ep.ztgt = c.ztgt; ep.v0 = (int)v0;
             ep.G = c.G; ep.G_ld = c.Vc;
             ep.eref = c.mref;
-            st = launch_gemm<EPI_CE_EXP, false, false>(p, ep, dev, stream);
+            st = sets == 2 ? launch_gemm<EPI_CE_EXP, false, false, 2>(p, ep, dev, stream)
+                           : launch_gemm<EPI_CE_EXP, false, false, 1>(p, ep, dev, stream);
             if (st != ATTT_OK) return st;
         }
         CeChunkArgs ca{};
-        ca.part = c.part; ca.ntiles = ntiles; ca.tile_w = plan.logits.BN; ca.L = (int)L; ca.V = (int)V;
+        ca.part = c.part; ca.ntiles = ntiles; ca.tile_w = width; ca.L = (int)L; ca.V = (int)V;
         ca.G = c.G; ca.G_ld = c.Vc;
         ca.aref = c.aref; ca.mref = c.mref; ca.lm = c.lm; ca.ls = c.ls;
         ca.alpha = c.alpha; ca.beta = c.beta; ca.gamma = c.gamma;

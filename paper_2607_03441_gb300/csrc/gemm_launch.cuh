@@ -167,10 +167,11 @@ inline uint32_t gemm_tmem_cols(int BN) {
 
 // `status` is the device word that records a timed-out wait; nullptr selects
 // the library's per-device status word.
-template <int EPI, bool A_MN, bool B_MN>
+template <int EPI, bool A_MN, bool B_MN, int SETS = 1>
 attt_status launch_gemm(const GemmProblem &p, const EpiParams &ep, int dev, cudaStream_t stream,
                         int *status = nullptr) {
     if (p.BN < 16 || p.BN > 256 || p.BN % 16 != 0) return ATTT_ERR_INVALID_ARG;
+    if (SETS == 2 && p.BN % 64 != 0) return ATTT_ERR_INVALID_ARG;  // sets of 32-column chunks
     if (B_MN && p.BN % 64 != 0) return ATTT_ERR_INVALID_ARG;
     if (p.pair && p.BN < 32) return ATTT_ERR_INVALID_ARG;  // BN/2 B rows per CTA (a multiple of 8)
     if (p.M <= 0 || p.N <= 0 || p.K <= 0) return ATTT_ERR_INVALID_ARG;
@@ -236,7 +237,7 @@ attt_status launch_gemm(const GemmProblem &p, const EpiParams &ep, int dev, cuda
     g.BN = p.BN;
     // B rows one CTA stages (whole 64-column boxes when MN-major)
     const int bn_cta = !p.pair ? p.BN : B_MN ? (int)round_up(p.BN / 2, 64) : p.BN / 2;
-    g.e_stage_bytes = (EPI == EPI_CE_EXP || EPI == EPI_BF16) ? kEStageBytes
+    g.e_stage_bytes = (EPI == EPI_CE_EXP || EPI == EPI_BF16) ? SETS * kEStageBytes
                       : (EPI == EPI_F32_ACC || EPI == EPI_F32_PART) ? kF32StageBytes
                       : EPI == EPI_KL                        ? kKlXBytes
                                                              : 0u;
@@ -290,7 +291,7 @@ attt_status launch_gemm(const GemmProblem &p, const EpiParams &ep, int dev, cuda
     const size_t smem = gemm_smem_bytes(bn_cta, g.stages, g.e_stage_bytes);
     const int ntiles = g.whole_tiles + (tiles - g.whole_tiles) * g.tail_s;  // work items
     cudaLaunchConfig_t cfg = {};
-    cfg.blockDim = dim3(p.pair ? kGemmPairThreads : kGemmThreads);
+    cfg.blockDim = dim3((unsigned)(p.pair ? gemm_pair_threads(SETS) : gemm_threads(SETS)));
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
@@ -302,7 +303,7 @@ attt_status launch_gemm(const GemmProblem &p, const EpiParams &ep, int dev, cuda
     }
     if (!p.pair) {
         if constexpr (EPI != EPI_KL) {  // EPI_KL runs on CTA pairs only
-            auto kern = tc_gemm_kernel<EPI, A_MN, B_MN>;
+            auto kern = tc_gemm_kernel<EPI, A_MN, B_MN, SETS>;
             if (!set_smem_limit(reinterpret_cast<const void *>(kern), smem, dev)) return ATTT_ERR_CUDA;
             cfg.gridDim = dim3((unsigned)(ntiles < sms ? ntiles : sms));
             cfg.attrs = attr;
@@ -310,7 +311,7 @@ attt_status launch_gemm(const GemmProblem &p, const EpiParams &ep, int dev, cuda
             if (cudaLaunchKernelEx(&cfg, kern, ta, tb, tc, ta2, tb2, g) != cudaSuccess) return ATTT_ERR_CUDA;
         }
     } else {
-        auto kern = tc_gemm_pair_kernel<EPI, A_MN, B_MN>;
+        auto kern = tc_gemm_pair_kernel<EPI, A_MN, B_MN, SETS>;
         if (!set_smem_limit(reinterpret_cast<const void *>(kern), smem, dev)) return ATTT_ERR_CUDA;
         const int pairs = ntiles < units ? ntiles : units;
         cfg.gridDim = dim3((unsigned)(2 * pairs));

@@ -9,9 +9,9 @@
 //     memory stages of 64-deep K blocks, 128-byte swizzled;
 //   * warp 1: allocates TMEM and issues tcgen05.mma (one thread), four
 //     M128 x N(BN) x K16 MMAs per stage, into one of two TMEM accumulators;
-//   * warps 2-5: epilogue, one accumulator row per thread (tcgen05.ld
-//     32x32b), overlapping the next tile's MMAs through the second
-//     accumulator.  The epilogue kinds fuse the work that follows the
+//   * warps 2-5 (and, for short K, four more on the other half of the columns):
+//     epilogue, one accumulator row per thread (tcgen05.ld 32x32b),
+//     overlapping the next tile's MMAs through the second accumulator.  The epilogue kinds fuse the work that follows the
 //     contraction so that nothing of size [M x N] goes back to HBM unless it
 //     is the result itself.
 // An operand is K-major (K contiguous in memory: a row-major [rows, K] matrix)
@@ -43,8 +43,8 @@ constexpr int kMaxProj = 8;
 struct EpiParams {
     // CE
     const int32_t *tgt;  // [M] target ids
-    float2 *part;        // [vocab tiles, M] (max, sum of exp) in log2 units
-    int tile0;           // vocab tile index of column 0 of this launch
+    float2 *part;        // [column sets of BN / SETS, M] (max, sum of exp) in log2 units
+    int tile0;           // column set of column 0 of this launch
     float *ztgt;         // [M] target logit
     const float *eref;   // [M] reference (log2 units) E is written against; nullptr: the tile max
     int v0;              // vocab id of column 0 of this launch
@@ -95,16 +95,23 @@ struct GemmArgs {
 };
 
 constexpr uint32_t kABytes = 128 * 64 * 2;  // one A stage: 128 rows x 64 bf16
-constexpr int kGemmThreads = 192;
-// The pair kernel runs a second TMA producer warp (warp 6): the two take
-// alternate stages (one issuing thread keeps about one stage in flight).
-constexpr int kGemmPairThreads = 224;
+// Epilogue warps: SETS (1 or 2) sets of four, a row of the accumulator per
+// thread, each set taking BN / SETS of a tile's columns.  One set needs 7 us for
+// a 256-column tile of the logits, as long as the MMAs of 21 K blocks; two sets
+// halve that where K is short (EPI_CE_EXP up to kTwoSetBlocks: 4,679 x 776 x
+// 63,517 850 -> 794 us) and cost 2.6% where the MMAs are the longer part (2,048 x
+// 3,584 x 152,064, at the power cap), so long K and the other results keep one.
+constexpr int kTwoSetBlocks = 24;
+// Warps: 0 TMA producer, 1 MMA, 2-5 epilogue, then (pair kernel) 6 a second
+// producer, the two taking alternate stages, then the second epilogue set.
+__host__ __device__ constexpr int gemm_threads(int sets) { return 64 + 128 * sets; }
+__host__ __device__ constexpr int gemm_pair_threads(int sets) { return 96 + 128 * sets; }
 
 __host__ __device__ inline uint32_t gemm_b_stage_bytes(int BN) { return (uint32_t)BN * 128u; }
 
 // EPI_CE_EXP stages E through shared memory: per epilogue warp two buffers of
 // 32 rows x 32 bf16 (64-byte swizzle), written out by TMA stores.
-constexpr uint32_t kEStageBytes = 4 * 2 * 32 * 64;
+constexpr uint32_t kEStageBytes = 4 * 2 * 32 * 64;  // per epilogue set
 
 __host__ __device__ inline size_t gemm_smem_bytes(int BN, int stages, uint32_t extra = 0) {
     return 1024 + (size_t)stages * (kABytes + gemm_b_stage_bytes(BN)) + extra + 8 * (2 * stages + 5) + 16;
@@ -351,27 +358,27 @@ __device__ __forceinline__ void bf16_tile_store(const GemmArgs &g, const CUtenso
     }
 }
 
-// tmE / sE: the E tensor map and this warp's staging buffers (EPI_CE_EXP).
-template <int EPI>
-__device__ __forceinline__ void epilogue_tile(const GemmArgs &g, int gm_base, int tn, int row, uint32_t taddr,
-                                              const CUtensorMap *tmE = nullptr, uint32_t sE = 0) {
+// tmE / sE: the E tensor map and this warp's staging buffers (EPI_CE_EXP); ec: the
+// blocks it has stored so far (consecutive blocks alternate buffers, also from
+// one tile to the next).
+template <int EPI, int SETS>
+__device__ __forceinline__ void epilogue_tile(const GemmArgs &g, int gm_base, int tn, int set, int row, uint32_t taddr,
+                                              const CUtensorMap *tmE, uint32_t sE, uint32_t &ec) {
     const int gm = gm_base + row;
     const bool rv = gm < g.M;
     const int n_base = tn * g.BN;
-    // Columns this tile owns: [n_base, n_tile) within the tile, [n_base, n_end)
-    // within the problem.  TMEM is read in chunks of 32 (or 16) columns, so a
-    // chunk may run past the tile when BN is not a multiple of it; nothing
-    // past n_tile is ever stored (it belongs to the next tile).
-    const int n_tile = n_base + g.BN;
-    const int n_end = min(g.N, n_tile);
+    // Columns of this set: [c0, c1) of the tile (a multiple of 32 wide), those
+    // before n_end within the problem.
+    const int c0 = set * (g.BN / SETS), c1 = c0 + g.BN / SETS;
+    const int n_end = min(g.N, n_base + c1);
     const EpiParams &ep = g.ep;
 
     if constexpr (EPI == EPI_CE_EXP) {
-        // One pass over the tile's columns against the row reference R
+        // One pass over the set's columns against the row reference R
         // (log2 units): E = exp2(z2 - R) rounded to bf16 into the gradient
-        // block (columns past N as zeros), the tile max m, the sum of the
+        // block (columns past N as zeros), the set's max m, the sum of the
         // unrounded exp2(z2 - R) and the target logit.  The pair stored is
-        // (m, sum of exp2(z2 - m)).  A row whose tile max exceeds R by more
+        // (m, sum of exp2(z2 - m)).  A row whose max here exceeds R by more
         // than kCeRefJump (or has no reference) takes a second pass that
         // writes E = exp2(z2 - m) instead; that pass is warp-wide because TMEM
         // loads are.
@@ -380,7 +387,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs &g, int gm_base, in
         const int lane = row & 31, y = gm - lane;
         float mx = -INFINITY, zt = 0.f, sr = 0.f;
         bool hit = false;
-        for (int c = 0; c < g.BN; c += 32) {
+        for (int c = c0; c < c1; c += 32) {
             float v[32];
             tmem_ld_x32(taddr + (uint32_t)c, v);
             const int col0 = n_base + c;
@@ -422,7 +429,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs &g, int gm_base, in
             // zeros past N (inside the tile) are stored too: the dh
             // contraction reads whole 64-column K blocks; rows past M are
             // clipped by the tensor map
-            e_block_store(tmE, sE, c >> 5, lane, pk, col0, y);
+            e_block_store(tmE, sE, (int)(ec++), lane, pk, col0, y);
         }
         const bool own = rv && !(mx - R <= kCeRefJump);
         float sm;
@@ -439,7 +446,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs &g, int gm_base, in
             if (lane == 0) bulk_wait<0>();
             __syncwarp();
             float so = 0.f;
-            for (int c = 0; c < g.BN; c += 32) {
+            for (int c = c0; c < c1; c += 32) {
                 float v[32];
                 tmem_ld_x32(taddr + (uint32_t)c, v);
                 const int col0 = n_base + c;
@@ -454,12 +461,12 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs &g, int gm_base, in
                     __nv_bfloat162 b = __floats2bfloat162_rn(e0, e1);
                     pk[i / 2] = *reinterpret_cast<uint32_t *>(&b);
                 }
-                e_block_store(tmE, sE, c >> 5, lane, pk, col0, y);
+                e_block_store(tmE, sE, (int)(ec++), lane, pk, col0, y);
             }
             if (own) sm = so;
         }
         if (rv) {
-            ep.part[(int64_t)(ep.tile0 + tn) * g.M + gm] = make_float2(mx, sm);
+            if (n_base + c0 < g.N) ep.part[(int64_t)(ep.tile0 + SETS * tn + set) * g.M + gm] = make_float2(mx, sm);
             if (hit) ep.ztgt[gm] = zt;
         }
     }
@@ -589,8 +596,8 @@ __device__ __forceinline__ void epilogue_piece_f32_acc(const GemmArgs &g, const 
 // The kernel
 // ---------------------------------------------------------------------------
 
-template <int EPI, bool A_MN, bool B_MN>
-__global__ void __launch_bounds__(kGemmThreads, 1)
+template <int EPI, bool A_MN, bool B_MN, int SETS>
+__global__ void __launch_bounds__(gemm_threads(SETS), 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                    const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmA2,
                    const __grid_constant__ CUtensorMap tmB2, const GemmArgs g) {
@@ -619,7 +626,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(tfull0 + 8 * a, 1);
-            mbar_init(tempty0 + 8 * a, 4);
+            mbar_init(tempty0 + 8 * a, 4 * SETS);
         }
         griddep_launch_dependents();
         mbar_init(drain0, 1);
@@ -752,12 +759,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             if (!mbar_wait(drain0, 0u, &no_abort)) record_error(g.status, ATTT_ERR_TIMEOUT);
         }
     } else {
-        // ---------------- epilogue (warps 2..5) ----------------
+        // ---------------- epilogue (warps 2..5, and 6..9) ----------------
         griddep_wait();  // what the epilogue reads or overwrites may come from the previous grid
-        const int q = warp & 3;
+        const int q = warp & 3, set = warp >= 6 ? 1 : 0;
+        const int ew = q + 4 * set;  // staging slot of this warp
         const int row = q * 32 + lane;
         F32Stage fst{smem_u32(sE) + (uint32_t)q * 8192u, smem_u32(sE) + 32768u + (uint32_t)q * 16u, 0u};
-        uint32_t bec = 0;  // EPI_BF16 boxes stored by this warp
+        uint32_t bec = 0;  // bf16 blocks stored by this warp (picks its staging buffer)
         int it = 0;
         for (int w = blockIdx.x; w < nwork; w += gridDim.x, ++it) {
             const Work wi = work_item(g, w, g.tiles_m);
@@ -765,8 +773,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             const uint32_t par = ((uint32_t)it >> 1) & 1u;
             int ok = 1;
             if (lane == 0) ok = mbar_wait(tfull0 + 8 * acc, par, abort_flag) ? 1 : 0;
-            // one decision for all four epilogue warps
-            ok = named_barrier_and(1, 128, __shfl_sync(0xffffffffu, ok, 0));
+            // one decision for all epilogue warps
+            ok = named_barrier_and(1, 128 * SETS, __shfl_sync(0xffffffffu, ok, 0));
             if (!ok) {
                 if (lane == 0) { *abort_flag = 1; record_error(g.status, ATTT_ERR_TIMEOUT); }
                 break;
@@ -789,10 +797,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                     f32_part_store(g, &tmC, fst, lane, w * 128 + 32 * q, min(g.N - wi.tn * g.BN, g.BN), taddr);
             } else if constexpr (EPI == EPI_BF16) {
                 const int gm = wi.tm * 128 + row;
-                bf16_tile_store(g, &tmC, smem_u32(sE) + (uint32_t)q * 4096u, bec, lane, gm - lane, wi.tn * g.BN,
+                bf16_tile_store(g, &tmC, smem_u32(sE) + (uint32_t)ew * 4096u, bec, lane, gm - lane, wi.tn * g.BN,
                                 min(g.N, (wi.tn + 1) * g.BN), taddr);
             } else {
-                epilogue_tile<EPI>(g, wi.tm * 128, wi.tn, row, taddr, &tmC, smem_u32(sE) + (uint32_t)q * 4096u);
+                epilogue_tile<EPI, SETS>(g, wi.tm * 128, wi.tn, set, row, taddr, &tmC, smem_u32(sE) + (uint32_t)ew * 4096u,
+                                   bec);
             }
             tc_fence_before();
             __syncwarp();
@@ -820,8 +829,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
 // a third less shared-memory traffic per FLOP than the single-CTA kernel.
 // ---------------------------------------------------------------------------
 
-template <int EPI, bool A_MN, bool B_MN>
-__global__ void __launch_bounds__(kGemmPairThreads, 1)
+template <int EPI, bool A_MN, bool B_MN, int SETS>
+__global__ void __launch_bounds__(gemm_pair_threads(SETS), 1)
     tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                    const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmA2,
                    const __grid_constant__ CUtensorMap tmB2, const GemmArgs g) {
@@ -856,7 +865,7 @@ __global__ void __launch_bounds__(kGemmPairThreads, 1)
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(tfull0 + 8 * a, 1);
-            mbar_init(tempty0 + 8 * a, 8);
+            mbar_init(tempty0 + 8 * a, 8 * SETS);
         }
         griddep_launch_dependents();
         mbar_init(drain0, 1);
@@ -1004,13 +1013,14 @@ __global__ void __launch_bounds__(kGemmPairThreads, 1)
             volatile int no_abort = 0;
             if (!mbar_wait(drain0, 0u, &no_abort)) record_error(g.status, ATTT_ERR_TIMEOUT);
         }
-    } else if (warp >= 2 && warp <= 5) {
-        // ---------------- epilogue (warps 2..5, both CTAs) ----------------
+    } else {
+        // ---------------- epilogue (warps 2..5 and 7..10, both CTAs) ----------------
         griddep_wait();  // what the epilogue reads or overwrites may come from the previous grid
-        const int q = warp & 3;
+        const int q = warp & 3, set = warp >= 7 ? 1 : 0;
+        const int ew = q + 4 * set;  // staging slot of this warp
         const int row = q * 32 + lane;
         F32Stage fst{smem_u32(sE) + (uint32_t)q * 8192u, smem_u32(sE) + 32768u + (uint32_t)q * 16u, 0u};
-        uint32_t bec = 0;  // EPI_BF16 boxes stored by this warp
+        uint32_t bec = 0;  // bf16 blocks stored by this warp (picks its staging buffer)
         uint32_t kl_ck = 0;  // EPI_KL chunks handed over by this warp pair
         int it = 0;
         for (int w = cid; w < nwork; w += ncl, ++it) {
@@ -1019,8 +1029,8 @@ __global__ void __launch_bounds__(kGemmPairThreads, 1)
             const uint32_t par = ((uint32_t)it >> 1) & 1u;
             int ok = 1;
             if (lane == 0) ok = mbar_wait(tfull0 + 8 * acc, par, abort_flag) ? 1 : 0;
-            // one decision for all four epilogue warps
-            ok = named_barrier_and(1, 128, __shfl_sync(0xffffffffu, ok, 0));
+            // one decision for all epilogue warps
+            ok = named_barrier_and(1, 128 * SETS, __shfl_sync(0xffffffffu, ok, 0));
             if (!ok) {
                 if (lane == 0) { *abort_flag = 1; record_error(g.status, ATTT_ERR_TIMEOUT); }
                 break;
@@ -1030,8 +1040,8 @@ __global__ void __launch_bounds__(kGemmPairThreads, 1)
             const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * g.BN);
             const int gm_base = wi.tm * 256 + 128 * (int)rank;
             if constexpr (EPI == EPI_KL) {
-                epilogue_kl(g, wi.tm * 128 + 64 * (int)rank, wi.tn, q, lane, taddr, reinterpret_cast<float *>(sE),
-                            kl_ck);
+                epilogue_kl(g, wi.tm * 128 + 64 * (int)rank, wi.tn, q, lane, taddr,
+                            reinterpret_cast<float *>(sE), kl_ck);
             } else if constexpr (EPI == EPI_F32_ACC) {
                 if (wi.piece >= 0) {
                     epilogue_piece_f32_acc(g, wi, gm_base, (int)rank, 2, row, taddr, &tmC, fst, abort_flag);
@@ -1047,10 +1057,11 @@ __global__ void __launch_bounds__(kGemmPairThreads, 1)
                     f32_part_store(g, &tmC, fst, lane, (w * 2 + (int)rank) * 128 + 32 * q,
                                    min(g.N - wi.tn * g.BN, g.BN), taddr);
             } else if constexpr (EPI == EPI_BF16) {
-                bf16_tile_store(g, &tmC, smem_u32(sE) + (uint32_t)q * 4096u, bec, lane, gm_base + 32 * q,
+                bf16_tile_store(g, &tmC, smem_u32(sE) + (uint32_t)ew * 4096u, bec, lane, gm_base + 32 * q,
                                 wi.tn * g.BN, min(g.N, (wi.tn + 1) * g.BN), taddr);
             } else {
-                epilogue_tile<EPI>(g, gm_base, wi.tn, row, taddr, &tmC, smem_u32(sE) + (uint32_t)q * 4096u);
+                epilogue_tile<EPI, SETS>(g, gm_base, wi.tn, set, row, taddr, &tmC, smem_u32(sE) + (uint32_t)ew * 4096u,
+                                   bec);
             }
             tc_fence_before();
             __syncwarp();
