@@ -283,6 +283,25 @@ def test_reference_jumps_over_chunks_and_narrow_tiles(attt, L, V, d):
         assert rel_l2(dh[rows[i]], rdh[i]) < DH_RL2, rows[i]
 
 
+@pytest.mark.parametrize("L,V,d", [(4400, 8000, 64), (8300, 600, 4096)])
+def test_row_tiles_in_groups(attt, L, V, d):
+    """Row tiles whose A exceeds half of L2 (E of the dh contraction in the first
+    shape, h of the logits in the second), so that they are walked in groups of
+    2,048 rows, the last one smaller: sampled rows of every group against the
+    oracle."""
+    h = wk.normal_bf16(L + 5, "h", (L, d), 1.0)
+    W = wk.normal_bf16(V + 5, "W", (V, d), 0.02)
+    rng = wk.rng_for(L + V + 5, "t")
+    tgt = rng.integers(0, V, L).astype(np.int32)
+    w = np.ones(L, np.float32)
+    _, dh, lse = _run(attt, h, W, tgt, w)
+    rows = np.unique(np.concatenate([np.arange(0, L, 1024), [L - 1], rng.choice(L, 8, replace=False)])).astype(np.int64)
+    rlse, _, rdh = oracle.ce_rows(h, W, tgt, w, rows)
+    np.testing.assert_allclose(lse[rows], rlse, atol=LSE_ATOL, rtol=0)
+    for i in range(len(rows)):
+        assert rel_l2(dh[rows[i]], rdh[i]) < DH_RL2, rows[i]
+
+
 def test_launch_counter_counts_every_kernel(attt):
     """One single-chunk call launches the reference kernel, GEMM1, the chunk
     kernel and GEMM2: four kernels, all counted."""
