@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(256) lora_prep_kernel(PrepArgs a) {
         }
         __syncthreads();
     }
-    const int64_t nB8 = (int64_t)a.rpad * a.dout[p] / 8;  // 16-byte vectors of BT_p
+    const int64_t nB8 = a.BT[p] ? (int64_t)a.rpad * a.dout[p] / 8 : 0;  // 16-byte vectors of BT_p (nullptr: not wanted)
     const int64_t rB8 = (int64_t)a.r * a.dout[p] / 8;     // of them copied from B_p (rows c < r)
     const int64_t ztk = (a.ntickets + a.nproj - 1) / a.nproj;  // this row's slice of the tickets
     const int64_t n = nB8 > ztk ? nB8 : ztk;
@@ -381,6 +381,18 @@ static double skinny_block(int nb, int n, bool mn) {
     return feed > issue ? feed : issue;
 }
 
+// A^T of the projections (K-major, rank padded to rpad) for ranks whose rows of
+// A are not 16-byte multiples, which TMA cannot read in place.
+static attt_status launch_prep_a(const attt_bf16 *const *d_A, int nproj, int64_t din, int r, int rpad,
+                                 __nv_bfloat16 *AT, int dev, cudaStream_t stream) {
+    PrepArgs a{};
+    for (int p = 0; p < nproj; ++p) a.A[p] = reinterpret_cast<const __nv_bfloat16 *>(d_A[p]);
+    a.nproj = nproj; a.r = r; a.rpad = rpad; a.din = din; a.AT = AT;
+    lora_prep_kernel<<<dim3(grid_for(cdiv(din, kPrepRows) * 256, 256, dev), nproj), 256, 0, stream>>>(a);
+    count_launch();
+    return cudaGetLastError() == cudaSuccess ? ATTT_OK : ATTT_ERR_CUDA;
+}
+
 // The most CTAs per tile (at most one per K block) with which `tiles` clusters
 // are resident together; 0 if the tiles alone are not.
 static int skinny_cluster(int64_t tiles, int64_t kb, int dev) {
@@ -487,9 +499,6 @@ static bool tmap_a_mn(CUtensorMap *m, const void *p, int64_t rows, int64_t k) {
     return make_tmap_bf16(m, p, (uint64_t)rows, (uint64_t)k, (uint64_t)rows * 2, 64, 64);
 }
 
-// s16[m, c] = bf16(scale sum_k a[m, k] M[k, c]) for c < rpad (zero past r): M =
-// A [din, r] read MN-major (mn) or M^T = B [r, dout] read K-major.  `zero`:
-// counters of the next launch.
 // Whether s u or s v takes the skinny form, and on how many CTAs per tile (0:
 // the grouped form).  Fewer than kSkinnyMinBlocks K blocks leave a cluster
 // nothing to split.  Measured at 2,048 x 3,584, r 16: grouped 15 us (and 4 us of
@@ -498,9 +507,13 @@ static int skinny_project_cluster(int64_t L, int64_t kb, int dev) {
     return kb < kSkinnyMinBlocks ? 0 : skinny_cluster(cdiv(L, 128), kb, dev);
 }
 
-static attt_status skinny_project(const attt_bf16 *d_a, const attt_bf16 *d_m, int64_t L, int64_t K, int r, int rpad,
-                                  bool mn, float scale, __nv_bfloat16 *s16, unsigned int *zero, int nzero, int c,
-                                  int dev, cudaStream_t stream) {
+// s16[m, c] = bf16(scale sum_k a[m, k] M[k, c]) for c < rpad (zero past r): M =
+// A [din, r] read MN-major (mn), or M^T read K-major: B [r, dout], or a prepared
+// A^T [rpad, din] (pdl: of the previous kernel).  `zero`: counters of the next
+// launch.
+static attt_status skinny_project(const attt_bf16 *d_a, const void *d_m, int64_t L, int64_t K, int r, int rpad,
+                                  bool mn, bool pdl, float scale, __nv_bfloat16 *s16, unsigned int *zero, int nzero,
+                                  int c, int dev, cudaStream_t stream) {
     SkinnyMaps maps;
     SkinnyArgs g{};
     if (!tmap_a(&maps.a[0], d_a, K, L)) return ATTT_ERR_INVALID_ARG;
@@ -514,7 +527,7 @@ static attt_status skinny_project(const attt_bf16 *d_a, const attt_bf16 *d_m, in
     s.nb = 1; s.n = rpad; s.b_mn = mn ? 1 : 0; s.kb = (int)cdiv(K, 64); s.N = rpad;
     s.out = GOUT_N16; s.alpha = scale; s.r = r; s.rpad = rpad; s.ld = rpad; s.out16 = s16;
     g.grp[0] = SkinnyGroup{0, c, 0, 1, (int)L, rpad, {}};
-    return launch_skinny<false>(maps, g, cdiv(L, 128), c, false, dev, stream);
+    return launch_skinny<false>(maps, g, cdiv(L, 128), c, pdl, dev, stream);
 }
 
 // How the passes of attt_lora_grad run as skinny launches: the clusters of each
@@ -530,9 +543,10 @@ static SkinnyGradPlan skinny_grad_plan(int64_t L, int64_t din, int nproj, const 
                                        int dev) {
     SkinnyGradPlan p{0, 0, 1, true};
     const int Nu = nproj * rpad;
-    if (r % 8 != 0 || nproj > kSkinnyMaxProj || Nu > kSkinnyMaxCols) return p;
+    if (nproj > kSkinnyMaxProj || Nu > kSkinnyMaxCols) return p;
     const int64_t rows = cdiv(L, 128), ku = cdiv(din, 64), kl = cdiv(L, 64);
-    const double bu = skinny_block(nproj, rpad, true), bv = skinny_block(1, rpad, false);
+    const double bu = r % 8 == 0 ? skinny_block(nproj, rpad, true) : skinny_block(1, Nu, false);
+    const double bv = skinny_block(1, rpad, false);
     int64_t kt = ku, kmin = ku, kmax = 0;
     for (int q = 0; q < nproj; ++q) {
         const int64_t k = cdiv(dout[q], 64);
@@ -575,6 +589,9 @@ static SkinnyGradPlan skinny_grad_plan(int64_t L, int64_t din, int nproj, const 
     // grouped against skinny: L 2,048, q and v at r 16, +2.7: 27.0 -> 22.3 us; L
     // 4,096, 14,336 -> 4,096 at r 32, +4.7: 63 -> 54; L 8,192, 4,096 -> 4,096 and
     // 1,024 at r 8, +5.4: 58 -> 64; L 6,000, three projections at r 32, +12: 74 -> 85).
+    // A rank that is not a multiple of 8 keeps a prep launch (A alone) in both
+    // forms; the same line serves it: 40 drawn groups of ranks 4 and 12, mean 31.0
+    // us grouped, 25.9 with this line, 26.7 with one 3.5 us lower.
     const int BN = Nu;  // every block of the grouped form carries this many B rows
     int64_t t2n = cdiv(din, 128);
     for (int q = 0; q < nproj; ++q) t2n += cdiv(dout[q], 128);
@@ -583,8 +600,8 @@ static SkinnyGradPlan skinny_grad_plan(int64_t L, int64_t din, int nproj, const 
     return p;
 }
 
-// Both passes of attt_lora_grad as skinny launches (two launches, the adapters
-// read in place).  r is a multiple of 8 (rows of A are 16-byte multiples).
+// Both passes of attt_lora_grad as skinny launches: the adapters are read in
+// place, A of a rank that is not a multiple of 8 after a launch that transposes it.
 static attt_status lora_grad_skinny(const attt_bf16 *d_x, int64_t L, int64_t din, int nproj,
                                     const attt_bf16 *const *d_dy, const int64_t *dout, const attt_bf16 *const *d_A,
                                     const attt_bf16 *const *d_B, int r, float scale, float *const *d_dA,
@@ -594,12 +611,20 @@ static attt_status lora_grad_skinny(const attt_bf16 *d_x, int64_t L, int64_t din
         SkinnyMaps maps;
         SkinnyArgs g{};
         g.status = status;
-        if (!tmap_a(&maps.a[0], d_x, din, L)) return ATTT_ERR_INVALID_ARG;
+        const bool mn = r % 8 == 0;  // rows of A are 16-byte multiples
+        if (!mn) {
+            const attt_status st = launch_prep_a(d_A, nproj, din, r, c.rpad, c.AT, dev, stream);
+            if (st != ATTT_OK) return st;
+        }
+        if (!tmap_a(&maps.a[0], d_x, din, L) ||
+            (!mn && !make_tmap_bf16(&maps.b[0], c.AT, (uint64_t)din, (uint64_t)c.Nu, (uint64_t)din * 2, 64,
+                                    (uint32_t)c.Nu)))
+            return ATTT_ERR_INVALID_ARG;
         SkinnySeg &u = g.seg[0];
-        u.nb = nproj; u.n = c.rpad; u.b_mn = 1; u.kb = (int)cdiv(din, 64); u.N = c.Nu;
+        u.nb = mn ? nproj : 1; u.n = mn ? c.rpad : c.Nu; u.b_mn = mn ? 1 : 0; u.kb = (int)cdiv(din, 64); u.N = c.Nu;
         u.out = GOUT_T16; u.alpha = 1.0f; u.out16 = c.uT16; u.ld = c.Lp; u.r = u.rpad = c.rpad;
         for (int p = 0; p < nproj; ++p) {
-            if (!make_tmap_bf16(&maps.b[p], d_A[p], (uint64_t)r, (uint64_t)din, (uint64_t)r * 2, 64, 64) ||
+            if ((mn && !make_tmap_bf16(&maps.b[p], d_A[p], (uint64_t)r, (uint64_t)din, (uint64_t)r * 2, 64, 64)) ||
                 !tmap_a(&maps.a[1 + p], d_dy[p], dout[p], L) ||
                 !make_tmap_bf16(&maps.b[nproj + p], d_B[p], (uint64_t)dout[p], (uint64_t)r, (uint64_t)dout[p] * 2, 64,
                                 (uint32_t)c.rpad))
@@ -610,6 +635,8 @@ static attt_status lora_grad_skinny(const attt_bf16 *d_x, int64_t L, int64_t din
             v.out = GOUT_T16; v.alpha = 1.0f; v.out16 = c.vT16 + (size_t)p * c.rpad * c.Lp; v.ld = c.Lp;
             v.r = v.rpad = c.rpad;
         }
+        if (!mn)  // slots nproj.. hold the B_p; those of the A_p after the first are unused
+            for (int p = 1; p < nproj; ++p) maps.b[p] = maps.b[0];
         g.nmaps_a = 1 + nproj; g.nmaps_b = 2 * nproj;
         const int rows = (int)cdiv(L, 128);
         if (pl.merged) {
@@ -620,7 +647,7 @@ static attt_status lora_grad_skinny(const attt_bf16 *d_x, int64_t L, int64_t din
             for (int q = 0; q < g.ngroup; ++q)
                 g.grp[q] = SkinnyGroup{q * rows, pl.c1, q, 1, (int)L, q == 0 ? c.Nu : c.rpad, {}};
         }
-        const attt_status st = launch_skinny<false>(maps, g, (int64_t)rows * g.ngroup, pl.c1, false, dev, stream);
+        const attt_status st = launch_skinny<false>(maps, g, (int64_t)rows * g.ngroup, pl.c1, !mn, dev, stream);
         if (st != ATTT_OK) return st;
     }
     // pass 2, a tile per 128 columns of x (dA of every p) and of each dy_p (dB_p, stored transposed)
@@ -1114,9 +1141,14 @@ attt_status attt_lora_forward(const attt_bf16 *d_x, const attt_bf16 *d_W0, const
     st = current_device(&dev);
     if (st != ATTT_OK) return st;
     ProjLayout c = proj_layout(d_ws, L, din, dout, r, true);
-    const int cs = r % 8 == 0 ? skinny_project_cluster(L, cdiv(din, 64), dev) : 0;
-    if (cs > 0) {  // s u = s x A, A read in place
-        st = skinny_project(d_x, d_A, L, din, r, c.rpad, true, scale, c.s16, nullptr, 0, cs, dev, stream);
+    const int cs = skinny_project_cluster(L, cdiv(din, 64), dev);
+    if (cs > 0) {  // s u = s x A, A read in place where its rows allow it
+        const bool mn = r % 8 == 0;
+        if (!mn) st = launch_prep_a(&d_A, 1, din, r, c.rpad, c.AT, dev, stream);
+        if (st != ATTT_OK) return st;
+        st = mn ? skinny_project(d_x, d_A, L, din, r, c.rpad, true, false, scale, c.s16, nullptr, 0, cs, dev, stream)
+                : skinny_project(d_x, c.AT, L, din, c.rpad, c.rpad, false, true, scale, c.s16, nullptr, 0, cs, dev,
+                                 stream);
         if (st != ATTT_OK) return st;
     } else {
     {   // A^T (and B) padded to rpad rows, tickets zeroed
@@ -1179,8 +1211,8 @@ attt_status attt_lora_input_grad(const attt_bf16 *d_dy, const attt_bf16 *d_W0, c
     ProjLayout c = proj_layout(d_ws, L, din, dout, r, false);
     const int cs = skinny_project_cluster(L, cdiv(dout, 64), dev);
     if (cs > 0) {  // s v = s dy B^T, and the tail split's counters zeroed
-        st = skinny_project(d_dy, d_B, L, dout, r, c.rpad, false, scale, c.s16, c.tickets + c.tiles, kDxSplitRegions,
-                            cs, dev, stream);
+        st = skinny_project(d_dy, d_B, L, dout, r, c.rpad, false, false, scale, c.s16, c.tickets + c.tiles,
+                            kDxSplitRegions, cs, dev, stream);
         if (st != ATTT_OK) return st;
     } else {
         if (cudaMemsetAsync(c.tickets, 0, sizeof(unsigned int) * (size_t)(c.tiles + kDxSplitRegions), stream) !=

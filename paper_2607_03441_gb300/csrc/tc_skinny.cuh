@@ -10,7 +10,8 @@
 // (the result does not depend on timing).  The adapters are read in place
 // (K-major B [r, dout] as rows of a tile, A [din, r] as an MN-major tile of
 // half-used 64-column boxes, zero-filled past r), so no kernel has to prepare
-// them.
+// them; only A of a rank that is not a multiple of 8 (TMA cannot read its rows)
+// is transposed first.
 //
 // Measured on GB300 (call times, grouped form against this one): gradients of
 // q and v of the 7B-class update (2,048 rows, r 16) 27.0 -> 22.3 us, of one

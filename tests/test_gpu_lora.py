@@ -180,6 +180,8 @@ def test_ragged_shapes_and_repeatability(attt, L, din, douts, r):
     (1300, 640, [1288], 64),                  # 64 columns
     (2100, 3584, [3584, 512], 16),            # u and v of a row tile on one cluster
     (1000, 648, [2992, 1584, 3808, 1792], 32),  # two dB tiles share a cluster beside the wider dA tiles
+    (200, 1544, [776, 2056], 12),             # rank not a multiple of 8: A transposed first, one u operand
+    (130, 2056, [1032], 3),                   # an odd rank
 ])
 def test_tiles_on_clusters(attt, L, din, douts, r):
     """Groups whose tiles are few enough for clusters that split their K blocks

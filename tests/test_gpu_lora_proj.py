@@ -129,3 +129,17 @@ def test_planned_tiles(attt, shape):
     assert torch.equal(dx, attt.attt_lora_input_grad(bf16_dev(dy), *w))
     assert rel_l2(dx.cpu().numpy()[rows], oracle.lora_input_grad(dy[rows], W0, A, B, s)) < DX_RL2
     assert attt.attt_device_status() == 0
+
+
+@pytest.mark.parametrize("shape", [(70, 1032, 520, 12), (300, 2056, 1544, 5)])
+def test_forward_at_ranks_without_aligned_rows(attt, shape):
+    """Ranks that are not multiples of 8: A is transposed first, then s u runs
+    on clusters as for the others."""
+    L, din, dout, r = shape
+    x, _, W0, A, B = _inputs(L + din + r, L, din, dout, r)
+    w = (bf16_dev(W0), bf16_dev(A), bf16_dev(B), 2.0)
+    h = attt.attt_lora_forward(bf16_dev(x), *w)
+    assert torch.equal(h, attt.attt_lora_forward(bf16_dev(x), *w))
+    rows = _rows(L, 20, L)
+    assert rel_l2(h.float().cpu().numpy()[rows], oracle.lora_forward(x[rows], W0, A, B, 2.0)) < H_RL2
+    assert attt.attt_device_status() == 0
