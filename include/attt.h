@@ -353,7 +353,9 @@ ATTT_API size_t attt_lora_input_grad_workspace_bytes(int64_t L, int64_t din, int
  * rounded to bf16 once; products are bf16, sums fp32.  Requirements:
  * L >= 1, din and dout multiples of 8 (>= 8), 1 <= r <= 64, every pointer
  * 16-byte aligned, d_ws at least attt_lora_forward_workspace_bytes(L, din,
- * dout, r) bytes and 256-byte aligned.  Three launches.
+ * dout, r) bytes and 256-byte aligned.  Two to four launches: s (x A) (and A
+ * transposed before it where its rows cannot be read in place), the
+ * contraction, and the sum of its K pieces where few tiles are cut.
  */
 ATTT_API attt_status attt_lora_forward(const attt_bf16 *d_x, const attt_bf16 *d_W0, const attt_bf16 *d_A,
                                        const attt_bf16 *d_B, int64_t L, int64_t din, int64_t dout, int r,
@@ -365,7 +367,8 @@ ATTT_API attt_status attt_lora_forward(const attt_bf16 *d_x, const attt_bf16 *d_
  * [L, dout]) of its output:  dx = dy W0^T + s (dy B^T) A^T  (fp32 [L, din]
  * into d_dx).  Shapes and alignment as attt_lora_forward; r must be a
  * multiple of 8 (A is read in place; ATTT_ERR_UNSUPPORTED otherwise).
- * s (dy B^T) is rounded to bf16 once.  Two launches.
+ * s (dy B^T) is rounded to bf16 once.  Two or three launches (the third sums
+ * the contraction's K pieces where few tiles are cut).
  */
 ATTT_API attt_status attt_lora_input_grad(const attt_bf16 *d_dy, const attt_bf16 *d_W0, const attt_bf16 *d_A,
                                           const attt_bf16 *d_B, int64_t L, int64_t din, int64_t dout, int r,

@@ -49,8 +49,8 @@ struct CeLayout {
 };
 
 // Upper bound of the vocab chunk: the chunk's bf16 block E (L x Vc) is kept
-// near kCeEBytes (1 GB), so the workspace stays bounded whatever V is.  Each chunk costs
-// about 20 us of launch, ramp and tail on top of its FLOPs, and E is streamed
+// near kCeEBytes (1 GB), so the workspace stays bounded whatever V is.  Each
+// chunk costs about 20 us of launch, ramp and tail on top of its FLOPs, and E is streamed
 // once from L2 or HBM either way, so wider chunks are faster up to this bound
 // (d 3,584, V 152,064, one chunk against three: L 93 354 against 415 us, L 403
 // 660 against 796, L 2,048 2,350 against 2,390).

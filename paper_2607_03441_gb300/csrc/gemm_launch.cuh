@@ -128,7 +128,8 @@ inline TilePlan plan_tiles(int64_t M, int64_t N, int64_t kb, int sms, int64_t re
             if (pair && BN == 64) continue;
             const int64_t tiles = cdiv(M, rows) * cdiv(N, BN);
             // (pair tiles of 192 columns run their MMAs at 0.29 us a block, not 0.25)
-            const double mma = pair && BN == 192 ? 0.29e-6 : 128.0 * BN * 128 / kSmFlops, feed = block_feed_seconds(pair, BN, b_mn);
+            const double mma = pair && BN == 192 ? 0.29e-6 : 128.0 * BN * 128 / kSmFlops;
+            const double feed = block_feed_seconds(pair, BN, b_mn), block = mma > feed ? mma : feed;
             for (int64_t s = 1; s <= kMaxPieces; ++s) {
                 if (s > 1 && (kb < 16 * s || tiles * s * (rows / 128) * BN > regions * 256)) break;
                 double waves = (double)cdiv(tiles * s, units), extra = 0.0;
@@ -140,7 +141,7 @@ inline TilePlan plan_tiles(int64_t M, int64_t N, int64_t kb, int sms, int64_t re
                     }
                 }
                 if (s > 1) extra = kReduceFixed + kReduceByte * 8.0 * s * M * N;
-                const double t = waves * cdiv(kb, s) * (mma > feed ? mma : feed) + kTileFixed + BN * kTileColumn + extra;
+                const double t = waves * cdiv(kb, s) * block + kTileFixed + BN * kTileColumn + extra;
                 if (t < 0.98 * best_t) {  // the wider and whole forms at equal estimates
                     best_t = t;
                     best = TilePlan{pair != 0, BN, (int)s};

@@ -11,15 +11,16 @@
 // MMA side and the rank on N, so the tensor core streams x and dy once per
 // pass at HBM rate.  Reductions over L (or din/dout) are split across CTAs
 // (stream-K, tc_group.cuh) and summed in a fixed order by the piece that
-// finishes each tile last; u and v go to bf16 in between.  Three launches per
-// call: prep (adapters to K-major), pass 1 (u and every v_p, grouped), pass 2
-// (dA and every dB_p, grouped).
+// finishes each tile last; u and v go to bf16 in between.  Groups whose tiles
+// are few take two launches on clusters (tc_skinny.cuh; skinny_grad_plan), pass
+// 1 (u and every v_p) and pass 2 (dA and every dB_p), the adapters read in
+// place; the others three: prep (adapters to K-major) and both passes grouped.
 //
 // The adapted projection itself (for a chained update, where the projection
 // feeds the LM head): the forward h = x W0 + s (x A) B and the input gradient
 // dx = dy W0^T + s (dy B^T) A^T.  Each is one tcgen05 contraction whose K runs
 // over two operand pairs, [x | s u] [W0 ; B] and [dy | s v] [W0^T ; A^T], after
-// a skinny grouped launch that forms s u = s x A or s v = s dy B^T in bf16.
+// a skinny launch that forms s u = s x A or s v = s dy B^T in bf16.
 #include <atomic>
 #include <cmath>
 

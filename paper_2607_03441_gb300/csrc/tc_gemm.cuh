@@ -11,9 +11,9 @@
 //     M128 x N(BN) x K16 MMAs per stage, into one of two TMEM accumulators;
 //   * warps 2-5 (and, for short K, four more on the other half of the columns):
 //     epilogue, one accumulator row per thread (tcgen05.ld 32x32b),
-//     overlapping the next tile's MMAs through the second accumulator.  The epilogue kinds fuse the work that follows the
-//     contraction so that nothing of size [M x N] goes back to HBM unless it
-//     is the result itself.
+//     overlapping the next tile's MMAs through the second accumulator.  The
+//     epilogue kinds fuse the work that follows the contraction so that nothing
+//     of size [M x N] goes back to HBM unless it is the result itself.
 // An operand is K-major (K contiguous in memory: a row-major [rows, K] matrix)
 // or MN-major (rows contiguous: a row-major [K, rows] matrix); both are
 // loaded by TMA with the 128-byte swizzle that tcgen05 reads natively.
@@ -800,8 +800,8 @@ __global__ void __launch_bounds__(gemm_threads(SETS), 1)
                 bf16_tile_store(g, &tmC, smem_u32(sE) + (uint32_t)ew * 4096u, bec, lane, gm - lane, wi.tn * g.BN,
                                 min(g.N, (wi.tn + 1) * g.BN), taddr);
             } else {
-                epilogue_tile<EPI, SETS>(g, wi.tm * 128, wi.tn, set, row, taddr, &tmC, smem_u32(sE) + (uint32_t)ew * 4096u,
-                                   bec);
+                epilogue_tile<EPI, SETS>(g, wi.tm * 128, wi.tn, set, row, taddr, &tmC,
+                                         smem_u32(sE) + (uint32_t)ew * 4096u, bec);
             }
             tc_fence_before();
             __syncwarp();
@@ -950,7 +950,8 @@ __global__ void __launch_bounds__(gemm_pair_threads(SETS), 1)
                     if (!B_MN) {
                         tma_load_2d_pair(b_dst, pb, fb, kbk, brow);
                     } else {
-                        for (int b = 0; b < b_boxes; ++b) tma_load_2d_pair(b_dst + 8192 * b, pb, fb, brow + 64 * b, kbk);
+                        for (int b = 0; b < b_boxes; ++b)
+                            tma_load_2d_pair(b_dst + 8192 * b, pb, fb, brow + 64 * b, kbk);
                     }
                     if (++stage == S) { stage = 0; phase ^= 1u; }
                 }
@@ -1060,8 +1061,8 @@ __global__ void __launch_bounds__(gemm_pair_threads(SETS), 1)
                 bf16_tile_store(g, &tmC, smem_u32(sE) + (uint32_t)ew * 4096u, bec, lane, gm_base + 32 * q,
                                 wi.tn * g.BN, min(g.N, (wi.tn + 1) * g.BN), taddr);
             } else {
-                epilogue_tile<EPI, SETS>(g, gm_base, wi.tn, set, row, taddr, &tmC, smem_u32(sE) + (uint32_t)ew * 4096u,
-                                   bec);
+                epilogue_tile<EPI, SETS>(g, gm_base, wi.tn, set, row, taddr, &tmC,
+                                         smem_u32(sE) + (uint32_t)ew * 4096u, bec);
             }
             tc_fence_before();
             __syncwarp();
