@@ -14,7 +14,8 @@
 // finishes each tile last; u and v go to bf16 in between.  Groups whose tiles
 // are few take two launches on clusters (tc_skinny.cuh; skinny_grad_plan), pass
 // 1 (u and every v_p) and pass 2 (dA and every dB_p), the adapters read in
-// place; the others three: prep (adapters to K-major) and both passes grouped.
+// place; the others three: prep (adapters to K-major) and both passes grouped;
+// and some the first pass on clusters and the second grouped.
 //
 // The adapted projection itself (for a chained update, where the projection
 // feeds the LM head): the forward h = x W0 + s (x A) B and the input gradient
@@ -236,7 +237,7 @@ struct GroupSpec {
 // 64-column box per adapter) and columns.
 constexpr int kSkinnyMaxProj = 4, kSkinnyMaxCols = 192;
 constexpr int kSkinnyMinBlocks = 8;
-constexpr double kSkinnyExtra = 5.0;  // microseconds (skinny_grad_plan)
+constexpr double kSkinnyExtra = 5.0, kSkinnyFirst = 6.0;  // microseconds (skinny_grad_plan)
 constexpr int kGroupMinStages = 2;
 // Ring stages a grouped launch's shared-memory ring keeps when it can (the
 // stage shape: the most K blocks per stage that leaves this many).  Measured
@@ -534,7 +535,8 @@ static attt_status skinny_project(const attt_bf16 *d_a, const void *d_m, int64_t
 // How the passes of attt_lora_grad run as skinny launches: the clusters of each
 // pass; whether pass 1 gives u and every v_p of a row tile to one cluster
 // (merged) or to one each; and in pass 2, how many tiles of a dB_p share a
-// cluster (ratio) beside the wider dA tiles.  c1 = 0: the grouped stream-K form.
+// cluster (ratio) beside the wider dA tiles.  c2 = 0: pass 2 in the grouped stream-K form; c1 = 0:
+// both passes.
 struct SkinnyGradPlan {
     int c1, c2, ratio;
     bool merged;
@@ -597,11 +599,21 @@ static SkinnyGradPlan skinny_grad_plan(int64_t L, int64_t din, int nproj, const 
     int64_t t2n = cdiv(din, 128);
     for (int q = 0; q < nproj; ++q) t2n += cdiv(dout[q], 128);
     const double grouped = (double)(rows * kt + t2n * kl) * skinny_block(1, BN, false) / num_sms(dev);
-    if (p.c2 == 0 || t1 + t2 > grouped + kSkinnyExtra) p.c1 = 0;
+    if (p.c2 == 0 || t1 + t2 > grouped + kSkinnyExtra) {
+        // Pass 1 alone on clusters, before a grouped pass 2, still saves the prep
+        // launch.  It pays at ranks past 16, where that kernel moves more and the
+        // grouped pass carries the widest B in every block (grouped against this: L
+        // 8,192, 5,120 -> 5,120 at r 64, 88.7 -> 76.9 us; L 4,096, gate and up of
+        // 14,336 at r 32, 112 -> 105; L 7,436, two at r 32, 97 -> 91) and not at 16
+        // and below (L 5,506, four at r 16, 54 -> 57; L 6,290, three at r 8, 42 -> 50).
+        const double g1 = (double)(rows * kt) * skinny_block(1, BN, false) / num_sms(dev);
+        p.c2 = 0;  // (c2 > 0 means that both passes run on clusters)
+        if (rpad < 32 || t1 > g1 + kSkinnyFirst) p.c1 = 0;
+    }
     return p;
 }
 
-// Both passes of attt_lora_grad as skinny launches: the adapters are read in
+// Both passes of attt_lora_grad as skinny launches, or the first one: the adapters are read in
 // place, A of a rank that is not a multiple of 8 after a launch that transposes it.
 static attt_status lora_grad_skinny(const attt_bf16 *d_x, int64_t L, int64_t din, int nproj,
                                     const attt_bf16 *const *d_dy, const int64_t *dout, const attt_bf16 *const *d_A,
@@ -648,8 +660,12 @@ static attt_status lora_grad_skinny(const attt_bf16 *d_x, int64_t L, int64_t din
             for (int q = 0; q < g.ngroup; ++q)
                 g.grp[q] = SkinnyGroup{q * rows, pl.c1, q, 1, (int)L, q == 0 ? c.Nu : c.rpad, {}};
         }
+        if (pl.c2 == 0) {  // pass 2 is grouped: its counters start at zero
+            g.zero = c.tickets;
+            g.nzero = (int)c.tiles;
+        }
         const attt_status st = launch_skinny<false>(maps, g, (int64_t)rows * g.ngroup, pl.c1, !mn, dev, stream);
-        if (st != ATTT_OK) return st;
+        if (st != ATTT_OK || pl.c2 == 0) return st;
     }
     // pass 2, a tile per 128 columns of x (dA of every p) and of each dy_p (dB_p, stored transposed)
     SkinnyMaps maps;
@@ -701,12 +717,17 @@ attt_status lora_grad_run(const attt_bf16 *d_x, int64_t L, int64_t din, int npro
     LoraLayout c = lora_layout(d_ws, L, din, nproj, dout, r);
     const int BN = c.BN;
     const SkinnyGradPlan pl = skinny_grad_plan(L, din, nproj, dout, r, c.rpad, dev);
-    if (pl.c1 > 0)
+    if (pl.c2 > 0)
         return lora_grad_skinny(d_x, L, din, nproj, d_dy, dout, d_A, d_B, r, scale, d_dA, d_dB, c, pl, status, dev,
                                 stream);
+    if (pl.c1 > 0) {  // pass 1 alone
+        st = lora_grad_skinny(d_x, L, din, nproj, d_dy, dout, d_A, d_B, r, scale, d_dA, d_dB, c, pl, status, dev,
+                              stream);
+        if (st != ATTT_OK) return st;
+    }
 
-    // prep: adapters to K-major (rank padded with zeros), accumulators zeroed
-    {
+    // prep: adapters to K-major (rank padded with zeros), counters zeroed
+    if (pl.c1 == 0) {
         PrepArgs a{};
         int64_t maxn = cdiv(din, kPrepRows) * 256;  // the transpose slabs (one block each)
         for (int p = 0; p < nproj; ++p) {
@@ -726,7 +747,7 @@ attt_status lora_grad_run(const attt_bf16 *d_x, int64_t L, int64_t din, int npro
     }
 
     // pass 1: u^T = (x AT^T)^T and v_p^T = (dy_p BT_p^T)^T, fp32 sums then bf16
-    {
+    if (pl.c1 == 0) {
         GroupSpec sp[kMaxGroup];
         int n = 0;
         GroupSpec &u = sp[n++];

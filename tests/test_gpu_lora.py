@@ -182,6 +182,8 @@ def test_ragged_shapes_and_repeatability(attt, L, din, douts, r):
     (1000, 648, [2992, 1584, 3808, 1792], 32),  # two dB tiles share a cluster beside the wider dA tiles
     (200, 1544, [776, 2056], 12),             # rank not a multiple of 8: A transposed first, one u operand
     (130, 2056, [1032], 3),                   # an odd rank
+    (4200, 5000, [5128], 32),                 # pass 1 on clusters, pass 2 grouped
+    (4300, 5128, [4992], 20),                 # the same, A transposed first
 ])
 def test_tiles_on_clusters(attt, L, din, douts, r):
     """Groups whose tiles are few enough for clusters that split their K blocks
