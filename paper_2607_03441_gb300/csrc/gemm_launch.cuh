@@ -36,8 +36,8 @@ struct GemmProblem {
     float *split_ws = nullptr;
     unsigned int *split_tick = nullptr;
     int split_regions = 0;
-    // EPI_F32_PART: K pieces per tile; piece w (tile-major) stores its 128-row
-    // accumulators at row 128 w (pair: 256 w) of split_ws, BN columns wide.
+    // EPI_F32_PART: K pieces per tile; each stores its 128-row accumulators
+    // (pair: 256) at its part_row of split_ws, BN columns wide.
     int pieces = 1;
 };
 
@@ -150,6 +150,17 @@ inline TilePlan plan_tiles(int64_t M, int64_t N, int64_t kb, int sms, int64_t re
         }
     }
     return best;
+}
+
+// Tile order: with all row tiles walked per column tile, every wave streams
+// all of A (a_bytes); once A exceeds half of L2, groups of `group` tiles (2,048
+// rows; of rows_tile each) keep theirs there and a wave of 76 pair tiles reads 8
+// row and 9.5 column blocks instead of 32 and 2.4.  At 8,192 x 5,120 x
+// 152,064 the logits contractions read 2.6 instead of 5.2 GB from DRAM and the dh
+// contractions 5.8 instead of 9.7 (per chunk), the call at the power cap 15.9 ->
+// 15.0 ms; where A fits (4,096 x 4,096) the logits lose 1% by it.  0: no groups.
+inline int tile_group(int64_t M, int rows_tile, int group, double a_bytes) {
+    return a_bytes > 64e6 && cdiv(M, rows_tile) > 2 * group ? group : 0;
 }
 
 constexpr size_t kMaxSmem = 232448;  // 227 KB opt-in per CTA on sm_100-class parts
@@ -275,17 +286,9 @@ attt_status launch_gemm(const GemmProblem &p, const EpiParams &ep, int dev, cuda
     g.b_k_off = p.b_k_off;
     g.tmem_cols = gemm_tmem_cols(p.BN);
     g.operands_ready = !p.operands_ready ? 0 : p.second_waits ? 2 : 1;
-    // Tile order: with all row tiles walked per column tile, every wave streams
-    // all of A; once A exceeds half of L2, groups of 2,048 rows keep theirs there
-    // and a wave of 76 pair tiles reads 8 row and 9.5 column blocks instead of
-    // 32 and 2.4.  At 8,192 x 5,120 x 152,064 the logits contractions read 2.6
-    // instead of 5.2 GB from DRAM and the dh contractions 5.8 instead of 9.7 (per
-    // chunk), the call at the power cap 15.9 -> 15.0 ms; where A fits (4,096 x
-    // 4,096) the logits lose 1% by it.
     const int rows_tile = EPI == EPI_KL ? 128 : p.pair ? 256 : 128;
     const int group = EPI == EPI_KL ? 8 : 2048 / rows_tile;
-    const double a_bytes = 2.0 * p.M * p.K * (EPI == EPI_KL ? 2 : 1);
-    g.group_m = a_bytes > 64e6 && cdiv(p.M, rows_tile) > 2 * group ? group : 0;
+    g.group_m = tile_group(p.M, rows_tile, group, 2.0 * p.M * p.K * (EPI == EPI_KL ? 2 : 1));
     g.status = status ? status : device_status_word(dev);
     g.ep = ep;
 

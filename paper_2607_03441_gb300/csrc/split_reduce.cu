@@ -22,10 +22,9 @@ __global__ void __launch_bounds__(kReduceThreads) split_reduce_kernel(const Spli
     if (i >= (int64_t)a.M * n4) return;
     const int row = (int)(i / n4), col = (int)(i - (int64_t)row * n4) * 4;
     const int tn = col / a.BN;
-    const int64_t tile = (int64_t)tn * a.tiles_m + row / a.rows;
-    // piece p of the tile: `rows` rows of BN columns, at row (tile pieces + p) rows
-    const float4 *src = reinterpret_cast<const float4 *>(
-        a.part + ((tile * a.pieces) * a.rows + row % a.rows) * a.BN + (col - tn * a.BN));
+    // piece p of the tile: `rows` rows of BN columns from part_row(.., p, ..)
+    const int64_t y = part_row(row / a.rows, tn, a.tiles_m, 0, a.pieces, a.rows) + row % a.rows;
+    const float4 *src = reinterpret_cast<const float4 *>(a.part + y * a.BN + (col - tn * a.BN));
     const int64_t step = (int64_t)a.rows * a.BN / 4;
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4

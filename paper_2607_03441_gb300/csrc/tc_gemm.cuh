@@ -152,7 +152,7 @@ struct Work {
     int tm, tn, kb0, kb1, piece, tail;
 };
 
-__device__ __forceinline__ Work work_item(const GemmArgs &g, int w, int tiles_m) {
+__host__ __device__ __forceinline__ Work work_item(const GemmArgs &g, int w, int tiles_m) {
     Work k;
     int t = w;
     k.piece = -1;
@@ -169,7 +169,7 @@ __device__ __forceinline__ Work work_item(const GemmArgs &g, int w, int tiles_m)
     }
     if (g.group_m > 0) {  // groups of group_m row tiles, m fastest within a group
         const int per = g.group_m * g.tiles_n, gr = t / per, r = t - gr * per;
-        const int rows = min(g.group_m, tiles_m - gr * g.group_m);
+        const int left = tiles_m - gr * g.group_m, rows = left < g.group_m ? left : g.group_m;
         k.tn = r / rows;
         k.tm = gr * g.group_m + r - k.tn * rows;
         return k;
@@ -179,8 +179,16 @@ __device__ __forceinline__ Work work_item(const GemmArgs &g, int w, int tiles_m)
     return k;
 }
 
-__device__ __forceinline__ int work_count(const GemmArgs &g, int tiles_m) {
+__host__ __device__ __forceinline__ int work_count(const GemmArgs &g, int tiles_m) {
     return g.whole_tiles + (tiles_m * g.tiles_n - g.whole_tiles) * g.tail_s;
+}
+
+// EPI_F32_PART: first row of a piece's region in the matrix of partials, for
+// accumulators of `rows` rows.  A function of the tile and not of the order in
+// which the tiles are walked (work_item), so that the kernel that sums the
+// pieces finds them whatever that order is.
+__host__ __device__ __forceinline__ int64_t part_row(int tm, int tn, int tiles_m, int piece, int pieces, int rows) {
+    return (((int64_t)tn * tiles_m + tm) * pieces + piece) * rows;
 }
 
 constexpr float kLog2e = 1.4426950408889634f;
@@ -794,7 +802,9 @@ __global__ void __launch_bounds__(gemm_threads(SETS), 1)
                 }
             } else if constexpr (EPI == EPI_F32_PART) {
                 if (wi.tm * 128 + 32 * q < g.M)
-                    f32_part_store(g, &tmC, fst, lane, w * 128 + 32 * q, min(g.N - wi.tn * g.BN, g.BN), taddr);
+                    f32_part_store(g, &tmC, fst, lane,
+                                   (int)part_row(wi.tm, wi.tn, g.tiles_m, wi.piece, g.tail_s, 128) + 32 * q,
+                                   min(g.N - wi.tn * g.BN, g.BN), taddr);
             } else if constexpr (EPI == EPI_BF16) {
                 const int gm = wi.tm * 128 + row;
                 bf16_tile_store(g, &tmC, smem_u32(sE) + (uint32_t)ew * 4096u, bec, lane, gm - lane, wi.tn * g.BN,
@@ -1055,7 +1065,9 @@ __global__ void __launch_bounds__(gemm_pair_threads(SETS), 1)
                 }
             } else if constexpr (EPI == EPI_F32_PART) {
                 if (gm_base + 32 * q < g.M)
-                    f32_part_store(g, &tmC, fst, lane, (w * 2 + (int)rank) * 128 + 32 * q,
+                    f32_part_store(g, &tmC, fst, lane,
+                                   (int)part_row(wi.tm, wi.tn, tiles_m2, wi.piece, g.tail_s, 256) + 128 * (int)rank +
+                                       32 * q,
                                    min(g.N - wi.tn * g.BN, g.BN), taddr);
             } else if constexpr (EPI == EPI_BF16) {
                 bf16_tile_store(g, &tmC, smem_u32(sE) + (uint32_t)ew * 4096u, bec, lane, gm_base + 32 * q,

@@ -302,6 +302,25 @@ def test_row_tiles_in_groups(attt, L, V, d):
         assert rel_l2(dh[rows[i]], rdh[i]) < DH_RL2, rows[i]
 
 
+@pytest.mark.parametrize("L,V,d", [(4200, 32000, 512), (4097, 20000, 512), (4352, 20000, 520), (6000, 50257, 384)])
+def test_row_tiles_in_groups_and_pieces(attt, L, V, d):
+    """Grouped row tiles of a dh contraction that also runs in K pieces and is
+    more than one column tile wide (test_tile_plan.py asserts so), where the
+    order of the tiles is not that of the pieces' regions: sampled rows of
+    every row tile, all columns, against the oracle."""
+    h = wk.normal_bf16(L + 6, "h", (L, d), 1.0)
+    W = wk.normal_bf16(V + 6, "W", (V, d), 0.02)
+    rng = wk.rng_for(L + V + 6, "t")
+    tgt = rng.integers(0, V, L).astype(np.int32)
+    w = np.ones(L, np.float32)
+    _, dh, lse = _run(attt, h, W, tgt, w)
+    rows = np.unique(np.concatenate([np.arange(0, L, 256), [L - 1], rng.choice(L, 8, replace=False)])).astype(np.int64)
+    rlse, _, rdh = oracle.ce_rows(h, W, tgt, w, rows)
+    np.testing.assert_allclose(lse[rows], rlse, atol=LSE_ATOL, rtol=0)
+    for i in range(len(rows)):
+        assert rel_l2(dh[rows[i]], rdh[i]) < DH_RL2, rows[i]
+
+
 def test_launch_counter_counts_every_kernel(attt):
     """One single-chunk call launches the reference kernel, GEMM1, the chunk
     kernel and GEMM2: four kernels, all counted."""

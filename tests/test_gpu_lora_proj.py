@@ -143,3 +143,22 @@ def test_forward_at_ranks_without_aligned_rows(attt, shape):
     rows = _rows(L, 20, L)
     assert rel_l2(h.float().cpu().numpy()[rows], oracle.lora_forward(x[rows], W0, A, B, 2.0)) < H_RL2
     assert attt.attt_device_status() == 0
+
+
+@pytest.mark.parametrize("shape", [(4352, 14336, 512, 16), (4352, 512, 14336, 16), (4737, 6784, 320, 8)])
+def test_row_tiles_in_groups_and_pieces(attt, shape):
+    """Grouped row tiles of a contraction in K pieces, more than one column tile
+    wide (test_tile_plan.py asserts so; the forward of the first and last
+    shape, the input gradient of the second): a row of every row tile, all
+    columns, in both directions."""
+    L, din, dout, r = shape
+    x, dy, W0, A, B = _inputs(L + din + dout, L, din, dout, r)
+    w = (bf16_dev(W0), bf16_dev(A), bf16_dev(B), 2.0)
+    rows = np.unique(np.concatenate([np.arange(0, L, 256), [L - 1]]))
+    h = attt.attt_lora_forward(bf16_dev(x), *w).float().cpu().numpy()[rows]
+    dx = attt.attt_lora_input_grad(bf16_dev(dy), *w).cpu().numpy()[rows]
+    assert attt.attt_device_status() == 0
+    ref_h, ref_dx = oracle.lora_forward(x[rows], W0, A, B, 2.0), oracle.lora_input_grad(dy[rows], W0, A, B, 2.0)
+    for i in range(len(rows)):
+        assert rel_l2(h[i], ref_h[i]) < H_RL2, rows[i]
+        assert rel_l2(dx[i], ref_dx[i]) < DX_RL2, rows[i]
