@@ -106,10 +106,16 @@ static CeLayout ce_layout(void *ws, int64_t L, int64_t d, int64_t V) {
     return c;
 }
 
-// Merges two (max, sum) pairs of an online logsumexp in log2 units.
+// Merges two (max, sum) pairs of an online logsumexp in log2 units.  While the
+// max is -inf the sum means nothing but that it may be NaN (logits that are
+// all NaN have no max): sums are added then, so that a NaN reaches the row, and
+// a later finite max scales what else they held to 0.
 __device__ __forceinline__ void lse_merge(float &m, float &s, float m2, float s2) {
     const float mx = fmaxf(m, m2);
-    if (mx == -INFINITY) return;
+    if (mx == -INFINITY) {
+        s += s2;
+        return;
+    }
     s = s * exp2f(m - mx) + s2 * exp2f(m2 - mx);
     m = mx;
 }
@@ -223,7 +229,10 @@ __global__ void __launch_bounds__(kChunkWarps * 32) ce_chunk_kernel(const CeChun
                 p[k] = t + k * kStreams < a.ntiles ? __ldcg(a.part + (int64_t)(t + k * kStreams) * L + j)
                                                    : make_float2(-INFINITY, 0.f);
             const float mx = fmaxf(m, fmaxf(fmaxf(p[0].x, p[1].x), fmaxf(p[2].x, p[3].x)));
-            if (mx == -INFINITY) continue;
+            if (mx == -INFINITY) {  // as lse_merge
+                s += (p[0].y + p[1].y) + (p[2].y + p[3].y);
+                continue;
+            }
             s *= exp2f(m - mx);
 #pragma unroll
             for (int k = 0; k < 4; ++k) s += p[k].y * exp2f(p[k].x - mx);

@@ -46,17 +46,18 @@ static KlLayout kl_layout(void *ws, int64_t L, int64_t V) {
 
 // One row's five numbers over some of its tiles.  merge: M = max(m, m2), s = s
 // 2^(m-M) + s2 2^(m2-M), x the same with x, x2; a part without tiles (m2 =
-// -inf) adds nothing.
+// -inf, s2 = 0) adds nothing.  A tile whose logits are all NaN has m2 = -inf too,
+// and s2 NaN, which must reach the row.
 struct KlPart {
     float mp, sp, x, mq, sq;
     __device__ __forceinline__ void merge(const KlPart &o) {
-        if (o.mp != -INFINITY) {
+        if (o.mp != -INFINITY || o.sp != 0.f) {
             const float M = fmaxf(mp, o.mp), a = exp2f(mp - M), b = exp2f(o.mp - M);  // mp = -inf: a = 0
             sp = sp * a + o.sp * b;
             x = x * a + o.x * b;
             mp = M;
         }
-        if (o.mq != -INFINITY) {
+        if (o.mq != -INFINITY || o.sq != 0.f) {
             const float N = fmaxf(mq, o.mq);
             sq = sq * exp2f(mq - N) + o.sq * exp2f(o.mq - N);
             mq = N;

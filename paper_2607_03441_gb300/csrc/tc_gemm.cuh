@@ -444,9 +444,9 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs &g, int gm_base, in
         if (!own) {
             // sum against m from the sum against R; when R - m >= 100 every
             // term against R may have underflowed, and such a tile is below
-            // 2^-92 of the row's sum (R is at most the row max)
+            // 2^-92 of the row's sum (R is at most the row max); a NaN stays
             const float dd = R - mx;
-            sm = (dd < 100.f) ? sr * exp2f(dd) : (sr > 0.f ? exp2f(log2f(sr) + dd) : 1.f);
+            sm = (dd < 100.f) ? sr * exp2f(dd) : (sr == 0.f ? 1.f : exp2f(log2f(sr) + dd));
         }
         if (__any_sync(0xffffffffu, own)) {
             // the warp's blocks again, after the first pass's stores have

@@ -321,6 +321,29 @@ def test_row_tiles_in_groups_and_pieces(attt, L, V, d):
         assert rel_l2(dh[rows[i]], rdh[i]) < DH_RL2, rows[i]
 
 
+@pytest.mark.parametrize("L,V,d", [(64, 8193, 64), (64, 8225, 512), (300, 40001, 64), (64, 70000, 2048)])
+def test_nan_in_the_head_reaches_every_row(attt, L, V, d):
+    """The last row of the head is NaN and alone in its column set (of 32 to
+    256 columns; the last shape: in a set with others): lse, loss and dh are
+    NaN, not the values without that column.  A NaN in one hidden state stays
+    with its row."""
+    h = wk.normal_bf16(L + 7, "h", (L, d), 1.0)
+    W = wk.normal_bf16(V + 7, "W", (V, d), 0.05)
+    tgt = wk.rng_for(V + 7, "t").integers(0, V - 1, L).astype(np.int32)
+    w = np.ones(L, np.float32)
+    nan = wk.bf16_bits(np.array([np.nan], np.float32))[0]
+    bad = W.copy()
+    bad[V - 1] = nan
+    loss, dh, lse = _run(attt, h, bad, tgt, w)
+    assert np.isnan(loss) and np.isnan(lse).all() and np.isnan(dh).all()
+    h2 = h.copy()
+    h2[5] = nan
+    loss, dh, lse = _run(attt, h2, W, tgt, w)
+    others = np.arange(L) != 5
+    assert np.isnan(loss) and np.isnan(lse[5]) and np.isnan(dh[5]).all()
+    assert np.isfinite(lse[others]).all() and np.isfinite(dh[others]).all()
+
+
 def test_launch_counter_counts_every_kernel(attt):
     """One single-chunk call launches the reference kernel, GEMM1, the chunk
     kernel and GEMM2: four kernels, all counted."""

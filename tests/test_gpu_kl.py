@@ -108,3 +108,24 @@ def test_bad_arguments(attt):
     assert e.value.code == attt.ATTT_ERR_WORKSPACE
     with pytest.raises(ValueError):
         attt.attt_kl_drift(a, a[:3], W)
+
+
+@pytest.mark.parametrize("V", [257, 4097, 30000])
+def test_nan_in_the_head_reaches_every_row(attt, V):
+    """The last row of the head is NaN, alone in its 256-column tile (first two
+    sizes) or with others: KL and its mean are NaN, not the values without
+    that column.  A NaN in one state stays with its row."""
+    L, d = 40, 64
+    hp, hq, W = _inputs(V, L, d, V, 0.3)
+    nan = wk.bf16_bits(np.array([np.nan], np.float32))[0]
+    bad = W.copy()
+    bad[V - 1] = nan
+    kl, mean = attt.attt_kl_drift(bf16_dev(hp), bf16_dev(hq), bf16_dev(bad))
+    assert torch.isnan(kl).all() and torch.isnan(mean).all()
+    for h in (hp, hq):
+        keep = h[5].copy()
+        h[5] = nan
+        kl, mean = attt.attt_kl_drift(bf16_dev(hp), bf16_dev(hq), bf16_dev(W))
+        kl = kl.cpu().numpy()
+        assert np.isnan(kl[5]) and np.isfinite(np.delete(kl, 5)).all() and torch.isnan(mean).all()
+        h[5] = keep
