@@ -133,7 +133,8 @@ ATTT_API attt_status attt_history_destroy(attt_history *h);
 
 /*
  * Empties the history (an episode boundary: the adapter and the history are
- * reset between episodes, Sec. 4 / Appendix C).  Async on `stream`.
+ * reset between episodes, Sec. 4 / Appendix C).  Async on `stream`, which may
+ * be a stream of any device, whichever device is current.
  */
 ATTT_API attt_status attt_history_reset(attt_history *h, attt_stream stream);
 
@@ -425,7 +426,7 @@ ATTT_API attt_status attt_wordsets_create(int max_updates, int64_t max_bytes, at
 /* Frees the sets and their device memory (synchronises the device). */
 ATTT_API attt_status attt_wordsets_destroy(attt_wordsets *s);
 
-/* Forgets every text (an episode boundary).  Async on `stream`. */
+/* Forgets every text (an episode boundary).  Async on `stream` (of any device). */
 ATTT_API attt_status attt_wordsets_reset(attt_wordsets *s, attt_stream stream);
 
 /*

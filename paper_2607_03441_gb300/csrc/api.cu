@@ -43,20 +43,34 @@ int pending_fault() {
     return f;
 }
 
+// A driver entry point, or nullptr.
+void *driver_fn(const char *name) {
+    void *fn = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion(name, &fn, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess)
+        return nullptr;
+    return fn;
+}
+
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     std::lock_guard<std::mutex> lk(g_mu);
-    if (!g_encode) {
-        void *fn = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            g_encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
-    }
+    if (!g_encode)
+        g_encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(driver_fn("cuTensorMapEncodeTiled"));
     return g_encode;
 }
 
 }  // namespace
+
+bool stream_is_current(cudaStream_t stream, int dev) {
+    // The contexts are compared: cudaStreamGetDevice ends a capture.
+    static const auto stream_ctx = reinterpret_cast<CUresult (*)(CUstream, CUcontext *)>(driver_fn("cuStreamGetCtx"));
+    static const auto current_ctx = reinterpret_cast<CUresult (*)(CUcontext *)>(driver_fn("cuCtxGetCurrent"));
+    int cur = -1;
+    CUcontext a = nullptr, b = nullptr;
+    return stream_ctx && current_ctx && cudaGetDevice(&cur) == cudaSuccess && cur == dev &&
+           stream_ctx(stream, &a) == CUDA_SUCCESS && current_ctx(&b) == CUDA_SUCCESS && a == b && a;
+}
 
 void count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 

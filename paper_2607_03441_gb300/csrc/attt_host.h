@@ -15,6 +15,10 @@ namespace attt {
 // ATTT_ERR_UNSUPPORTED / ATTT_ERR_CUDA.
 attt_status current_device(int *dev);
 
+// Whether `dev` is the current device and `stream` one of its streams (legal
+// during a capture; false where that cannot be told).
+bool stream_is_current(cudaStream_t stream, int dev);
+
 // Number of SMs of a device (cached).
 int num_sms(int dev);
 
@@ -58,9 +62,9 @@ attt_status ngram_weights_batch(attt_history *const *hs, int E, const int32_t *d
 attt_status history_insert_batch(attt_history *const *hs, int E, const int32_t *d_tokens, const int64_t *off,
                                  cudaStream_t stream);
 
-// Zeroes a (and b, when not nullptr): 16-byte aligned, sizes multiples of 16
-// (ngram.cu).
-attt_status clear_tables(void *a, size_t a_bytes, void *b, size_t b_bytes, cudaStream_t stream);
+// Zeroes a (and b, when not nullptr) of device table_dev: 16-byte aligned, sizes
+// multiples of 16; on any current device and any stream (ngram.cu).
+attt_status clear_tables(int table_dev, void *a, size_t a_bytes, void *b, size_t b_bytes, cudaStream_t stream);
 
 // Eq. 10 as attt_weighted_ce_fwd_bwd, with per-row normalisers `row_scale`
 // (dh_j = w_j row_scale_j (...); nullptr: 1/L for every row) and the per-row

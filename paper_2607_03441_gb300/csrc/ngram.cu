@@ -241,12 +241,18 @@ static attt_status launch_dependent(void (*kern)(P...), dim3 grid, unsigned thre
     return cudaGetLastError() == cudaSuccess ? ATTT_OK : ATTT_ERR_CUDA;
 }
 
-attt_status clear_tables(void *a, size_t a_bytes, void *b, size_t b_bytes, cudaStream_t stream) {
+attt_status clear_tables(int table_dev, void *a, size_t a_bytes, void *b, size_t b_bytes, cudaStream_t stream) {
+    // A kernel runs on the current device, from one of its streams, and writes
+    // that device's memory; a reset asks for none of these, so any other call
+    // takes memsets, as do the tables of another device.
+    if (!stream_is_current(stream, table_dev)) {
+        if (cudaMemsetAsync(a, 0, a_bytes, stream) != cudaSuccess ||
+            (b && cudaMemsetAsync(b, 0, b_bytes, stream) != cudaSuccess))
+            return ATTT_ERR_CUDA;
+        return ATTT_OK;
+    }
     const int64_t na = (int64_t)(a_bytes / 16), nb = (int64_t)(b_bytes / 16);
-    int dev;
-    const attt_status st = current_device(&dev);
-    if (st != ATTT_OK) return st;
-    const int64_t want = cdiv(na > nb ? na : nb, 256 * 4), most = (int64_t)num_sms(dev) * 8;
+    const int64_t want = cdiv(na > nb ? na : nb, 256 * 4), most = (int64_t)num_sms(table_dev) * 8;
     return launch_dependent(clear_kernel, dim3((unsigned)(want < 1 ? 1 : want < most ? want : most)), 256, stream,
                             static_cast<uint4 *>(a), na, static_cast<uint4 *>(b), nb);
 }
@@ -451,7 +457,8 @@ attt_status attt_history_destroy(attt_history *h) {
 attt_status attt_history_reset(attt_history *h, attt_stream stream) {
     ATTT_NVTX_RANGE();
     if (!h) return ATTT_ERR_INVALID_ARG;
-    const attt_status st = attt::clear_tables(h->d_table, h->capacity * sizeof(attt::Slot), nullptr, 0, stream);
+    const attt_status st =
+        attt::clear_tables(h->device, h->d_table, h->capacity * sizeof(attt::Slot), nullptr, 0, stream);
     if (st != ATTT_OK) return st;
     h->len = 0;
     return ATTT_OK;

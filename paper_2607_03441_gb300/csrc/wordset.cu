@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(kInsThreads) repetition_kernel(RepArgs a) {
 }  // namespace
 
 struct attt_wordsets {
-    int max_updates, W, count;
+    int device, max_updates, W, count;
     int64_t arena_cap, len;
     uint8_t *d_arena;
     unsigned long long *d_keys, *d_masks;
@@ -332,6 +332,7 @@ attt_status attt_wordsets_create(int max_updates, int64_t max_bytes, attt_wordse
     if (st != ATTT_OK) return st;
     attt_wordsets *s = new (std::nothrow) attt_wordsets{};
     if (!s) return ATTT_ERR_CUDA;
+    s->device = dev;
     s->max_updates = max_updates;
     s->W = (max_updates + 63) / 64;
     s->arena_cap = max_bytes + max_updates;  // texts and one separator each
@@ -375,8 +376,8 @@ attt_status attt_wordsets_destroy(attt_wordsets *s) {
 attt_status attt_wordsets_reset(attt_wordsets *s, attt_stream stream) {
     ATTT_NVTX_RANGE();
     if (!s) return ATTT_ERR_INVALID_ARG;
-    const attt_status st = attt::clear_tables(s->d_keys, s->capacity * sizeof(unsigned long long), s->d_masks,
-                                              s->capacity * s->W * sizeof(unsigned long long), stream);
+    const attt_status st = attt::clear_tables(s->device, s->d_keys, s->capacity * sizeof(unsigned long long),
+                                              s->d_masks, s->capacity * s->W * sizeof(unsigned long long), stream);
     if (st != ATTT_OK) return st;
     s->len = 0;
     s->count = 0;

@@ -319,3 +319,28 @@ def test_long_probe_runs(attt, n):
     assert attt.attt_history_status(h) == 0
     h.close()
     np.testing.assert_array_equal(got, [oracle.count_naive(H, g) for g in q])
+
+
+def test_reset_and_refill_in_a_graph(attt):
+    """An episode boundary captured in a CUDA graph: reset, append, weights,
+    replayed three times, each replay from an emptied table."""
+    rng = np.random.default_rng(11)
+    H = rng.integers(0, 60, 700).astype(np.int32)
+    x = H[50:250].copy()
+    h = attt.attt_history_create(3, 1000)
+    hd, xd = i32_dev(H), i32_dev(x)
+    attt.attt_history_insert(h, hd)
+    out = torch.empty(len(x), dtype=torch.float32, device=DEV)
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        attt.attt_history_reset(h, stream=s)
+        attt.attt_history_insert(h, hd, stream=s)
+        attt.attt_ngram_weights(h, xd, 0.05, out=out, stream=s)
+    for _ in range(3):
+        out.zero_()
+        g.replay()
+        _assert_bit_exact(out.cpu().numpy(), oracle.ngram_weights(H, x, 3))
+    assert attt.attt_history_status(h) == 0
+    h.close()
