@@ -265,6 +265,15 @@ __global__ void __launch_bounds__(kSkinnyThreads, 1)
             if (!ok) {
                 *abort_flag = 1;
                 record_error(g.status, ATTT_ERR_TIMEOUT);
+                // The producer may have issued every load and gone: those that no MMA
+                // waited for (at most a ring of them) land before the CTA retires, as far
+                // as bounded waits of this thread's own can see to it.
+                volatile int no_abort = 0;
+                for (int i = 0; i < S && mbar_wait(full0 + 8 * slot, phase, &no_abort); ++i)
+                    if (++slot == S) {
+                        slot = 0;
+                        phase ^= 1u;
+                    }
             }
             umma_commit(done);
         }
