@@ -25,7 +25,10 @@
 namespace attt {
 
 constexpr int kCeBN = 256;
-constexpr int kCeMinSet = 32;     // columns of the narrowest set (half a 64-column tile) of the logits contraction
+// (max, sum) pairs of sets narrower than those of 256-column tiles, at most: the
+// plan takes narrow tiles only where few tiles would leave SMs idle (L 1 to
+// 20,000, V 256 to 262,144, d 64 to 8,192 on 152 SMs: at most 1,125,316 pairs).
+constexpr int64_t kCeNarrowPairs = 5ll << 18;  // 10 MB
 constexpr int kCeMaxTiles = 1024;  // chunk width at most, in kCeBN columns
 constexpr int kChunkWarps = 16;  // ce_chunk_kernel: 16 warps of 4 tiles x 8 rows
 constexpr int kChunkRows = 8;    // rows per block: lane & 7
@@ -70,11 +73,23 @@ struct CePlan {
     TilePlan logits, dh;
 };
 
+// Epilogue sets of a logits tile.
+static int ce_sets(int64_t d) { return cdiv(d, 64) <= kTwoSetBlocks ? 2 : 1; }
+
+// (max, sum) pairs that the sets of a chunk of Vc columns may need.
+static int64_t ce_pairs(int64_t L, int64_t d, int64_t Vc) {
+    const int64_t wide = cdiv(Vc, kCeBN) * ce_sets(d) * L, most = cdiv(Vc, 64) * ce_sets(d) * L;
+    const int64_t narrow = most < kCeNarrowPairs ? most : kCeNarrowPairs;
+    return wide > narrow ? wide : narrow;
+}
+
 static CePlan ce_plan(int64_t L, int64_t d, int64_t V, int regions, int sms) {
     CePlan p{};
     const int64_t nchunks = cdiv(V, ce_chunk_max(L, V));
     p.Vc = round_up(cdiv(V, nchunks), kCeBN);  // equal chunks
     p.logits = plan_tiles(L, p.Vc, cdiv(d, 64), sms, 0, false, false);
+    const int64_t pairs = ce_pairs(L, d, ce_chunk_max(L, V));
+    while (p.logits.BN < kCeBN && cdiv(p.Vc, p.logits.BN / ce_sets(d)) * L > pairs) p.logits.BN += 64;
     p.dh = plan_tiles(L, d, cdiv(p.Vc, 64), sms, regions, true, true);
     return p;
 }
@@ -88,7 +103,7 @@ static CeLayout ce_layout(void *ws, int64_t L, int64_t d, int64_t V) {
     c.Vc = ce_chunk_max(L, V);
     c.nblk = cdiv(L, kChunkRows);
     Carve cv{static_cast<char *>(ws), 0};
-    c.part = cv.take<float2>((size_t)(cdiv(c.Vc, kCeMinSet) * L));
+    c.part = cv.take<float2>((size_t)ce_pairs(L, d, c.Vc));
     c.ztgt = cv.take<float>((size_t)L);
     c.block_sums = cv.take<float>((size_t)c.nblk);
     c.aref = cv.take<float>((size_t)L);
@@ -425,7 +440,7 @@ attt_status ce_fwd_bwd_run(const attt_bf16 *d_h, const attt_bf16 *d_W, const int
     const CePlan plan = ce_plan(L, d, V, c.split_regions, num_sms(dev));
     for (int64_t v0 = 0, ci = 0; v0 < V; v0 += plan.Vc, ++ci) {
         const int64_t Nc = (V - v0 < plan.Vc) ? V - v0 : plan.Vc;
-        const int sets = cdiv(d, 64) <= kTwoSetBlocks ? 2 : 1;
+        const int sets = ce_sets(d);
         const int width = plan.logits.BN / sets;  // columns of a tile that one epilogue set takes
         const int ntiles = (int)cdiv(Nc, width);
         const bool last = v0 + Nc >= V;

@@ -51,6 +51,21 @@ def test_host_only_calls(lib_path):
     assert attt.attt_lora_workspace_bytes(256, 512, [512], 65) == 0
 
 
+@pytest.mark.parametrize("L,d,V", [(1, 512, 8192), (93, 3584, 152064), (2048, 3584, 152064), (2048, 1536, 152064),
+                                   (8192, 5120, 152064), (300, 512, 50257)])
+def test_eq10_workspace_holds_little_beside_the_block_and_the_pieces(lib_path, L, d, V):
+    """The bf16 block E, at most 320 regions of 128 KB of K pieces, a (max, sum)
+    pair per row and column set (128 columns, or 10 MB of narrower ones), row
+    terms."""
+    from paper_2607_03441_gb300 import attt
+    chunk = min(-(-V // 256) * 256, max(4096, (1 << 30) // (2 * L) // 256 * 256))
+    got = attt.attt_ce_workspace_bytes(L, d, V)
+    regions = min(320, 32 * -(-L // 256) * -(-d // 256))
+    pairs = max(chunk // (128 if d <= 1536 else 256) * L, min(5 << 18, chunk // (32 if d <= 1536 else 64) * L))
+    assert 2 * L * chunk < got <= 2 * L * chunk + regions * 131072 + 8 * pairs + 64 * L + 65536
+    assert attt.attt_ce_workspace_max_bytes(L, d, V) >= got
+
+
 def test_product_has_no_oracle_or_cpu_path():
     """Nothing on the product path imports the oracle or falls back to torch
     compute: the binding only marshals arguments to libattt."""
