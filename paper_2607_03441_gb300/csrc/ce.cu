@@ -30,6 +30,7 @@ constexpr int kCeBN = 256;
 // 20,000, V 256 to 262,144, d 64 to 8,192 on 152 SMs: at most 1,125,316 pairs).
 constexpr int64_t kCeNarrowPairs = 5ll << 18;  // 10 MB
 constexpr int kCeMaxTiles = 1024;  // chunk width at most, in kCeBN columns
+static_assert(kCeMaxTiles * kCeBN <= kCeMaxChunk, "the fp32 range of dh is argued for chunks of kCeMaxChunk columns");
 constexpr int kChunkWarps = 16;  // ce_chunk_kernel: 16 warps of 4 tiles x 8 rows
 constexpr int kChunkRows = 8;    // rows per block: lane & 7
 // fp32 partials of 128 x kCeBN (128 KB each) for the K pieces of the dh

@@ -195,9 +195,10 @@ constexpr float kLog2e = 1.4426950408889634f;
 
 // A CE tile whose max exceeds the row reference by more than kCeRefJump
 // (log2 units) writes E against its own max instead, so E <= 2^64.  The dh
-// contraction of a chunk sums at most 2^16 such terms times |W|, and the fp32
-// accumulator holds that for |W| up to 2^40.
+// contraction of a chunk sums at most kCeMaxChunk = 2^18 such terms times |W|,
+// and the fp32 accumulator holds that for |W| up to 2^40 (2^122).
 constexpr float kCeRefJump = 64.f;
+constexpr int kCeMaxChunk = 1 << 18;
 
 // Per-row terms of EPI_F32_ACC for output row gm: ra, rb and, when the
 // epilogue subtracts gamma_m W[t_m, :], gamma and that row of W.
