@@ -435,8 +435,11 @@ static void skinny_split(const SkinnyArgs &g, SkinnyGroup &gr) {
 
 // Launches the groups of g (its groups, segments, tiles and columns filled in)
 // on `clusters` clusters of `c` CTAs.  `pdl`: a programmatic dependent of the
-// previous kernel.  False in *fits (nothing launched) if the accumulators of a
-// tile exceed TMEM or shared memory.
+// previous kernel.  The accumulators of a tile fit TMEM and, as partials, shared
+// memory whatever the call: the most columns are u and every v_p of a row tile
+// on one cluster, 2 kSkinnyMaxCols.
+constexpr uint32_t kSkinnyRingMax = ((uint32_t)kMaxSmem - 2048u) / 1024u * 1024u;
+static_assert(2 * kSkinnyMaxCols <= 512 && 2 * kSkinnyMaxCols * 512u <= kSkinnyRingMax, "accumulators of a tile");
 template <bool A_MN>
 static attt_status launch_skinny(const SkinnyMaps &maps, SkinnyArgs &g, int64_t clusters, int c, bool pdl, int dev,
                                  cudaStream_t stream) {
@@ -456,11 +459,10 @@ static attt_status launch_skinny(const SkinnyMaps &maps, SkinnyArgs &g, int64_t 
             if ((uint32_t)kb * b > ring) ring = (uint32_t)kb * b;
         }
     }
-    const uint32_t bound = ((uint32_t)kMaxSmem - 2048u) / 1024u * 1024u;
     g.cluster = c;
-    g.ring_bytes = ring < bound ? ring : bound;
+    g.ring_bytes = ring < kSkinnyRingMax ? ring : kSkinnyRingMax;
     if ((uint32_t)ncols * 512u > g.ring_bytes) g.ring_bytes = (uint32_t)ncols * 512u;
-    if (g.ring_bytes > bound || ncols > 512) return ATTT_ERR_INVALID_ARG;
+    if (g.ring_bytes > kSkinnyRingMax || ncols > 512) return ATTT_ERR_INVALID_ARG;
     g.tmem_cols = 32;
     while ((int)g.tmem_cols < ncols) g.tmem_cols <<= 1;
     if (!g.status) g.status = device_status_word(dev);
