@@ -148,14 +148,20 @@ def _check(code: int, where: str) -> None:
         raise AtttError(code, where)
 
 
+# torch's own way to a stream's handle; not public, so it may be missing
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream: Optional[torch.cuda.Stream]) -> int:
     """The cudaStream_t of `stream`, or of the current stream (asked for by its
-    handle: building a torch Stream object takes longer than a launch)."""
+    handle where torch has that: building a torch Stream object takes longer
+    than a launch)."""
     if stream is not None:
         return stream.cuda_stream
-    if not torch.cuda.is_initialized():
+    if _raw_stream is None or _raw_device is None or not torch.cuda.is_initialized():
         return torch.cuda.current_stream().cuda_stream
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return _raw_stream(_raw_device())
 
 
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:

@@ -4,6 +4,7 @@ import ctypes
 import os
 import re
 import subprocess
+import sys
 
 import pytest
 
@@ -64,6 +65,17 @@ def test_eq10_workspace_holds_little_beside_the_block_and_the_pieces(lib_path, L
     pairs = max(chunk // (128 if d <= 1536 else 256) * L, min(5 << 18, chunk // (32 if d <= 1536 else 64) * L))
     assert 2 * L * chunk < got <= 2 * L * chunk + regions * 131072 + 8 * pairs + 64 * L + 65536
     assert attt.attt_ce_workspace_max_bytes(L, d, V) >= got
+
+
+def test_current_stream_without_torch_internals():
+    """The binding finds the current stream's handle where torch lacks the
+    internal call for it."""
+    probe = ("import types, torch; del torch._C._cuda_getCurrentRawStream\n"
+             "from paper_2607_03441_gb300 import attt\n"
+             "torch.cuda.is_initialized = lambda: True\n"
+             "torch.cuda.current_stream = lambda: types.SimpleNamespace(cuda_stream=77)\n"
+             "assert attt._stream(None) == 77")
+    subprocess.run([sys.executable, "-c", probe], cwd=ROOT, check=True)
 
 
 def test_product_has_no_oracle_or_cpu_path():
