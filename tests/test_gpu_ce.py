@@ -242,8 +242,9 @@ def test_tail_pieces_deterministic(attt, L, V, d):
 def test_every_tile_in_pieces(attt, L, V, d):
     """Few rows, so every tile of the dh contraction runs as K pieces that a
     second kernel sums (64- to 256-column tiles, single CTAs and pairs, rows
-    and columns that end inside a tile): every row against the oracle at the
-    tolerances above, and two calls give the same bits."""
+    and columns that end inside a tile): the loss and every row, each by
+    itself, against the oracle at the tolerances above, and two calls give the
+    same bits."""
     h = wk.normal_bf16(L + 3, "h", (L, d), 1.0)
     W = wk.normal_bf16(V + 3, "W", (V, d), 0.05)
     rng = wk.rng_for(L + V + 3, "t")
@@ -254,10 +255,11 @@ def test_every_tile_in_pieces(attt, L, V, d):
     assert loss == loss2
     np.testing.assert_array_equal(dh.view(np.uint32), dh2.view(np.uint32))
     np.testing.assert_array_equal(lse.view(np.uint32), lse2.view(np.uint32))
-    rows = np.unique(np.concatenate([[0, L - 1], rng.choice(L, min(L, 12), replace=False)])).astype(np.int64)
-    rlse, _, rdh = oracle.ce_rows(h, W, tgt, w, rows)
-    np.testing.assert_allclose(lse[rows], rlse, atol=LSE_ATOL, rtol=0)
-    assert rel_l2(dh[rows], rdh) < DH_RL2
+    rloss, rlse, _, rdh = oracle.ce_loss(h, W, tgt, w)
+    assert abs(loss - rloss) <= LOSS_RTOL * abs(rloss), (loss, rloss)
+    np.testing.assert_allclose(lse, rlse, atol=LSE_ATOL, rtol=0)
+    for j in range(L):
+        assert rel_l2(dh[j], rdh[j]) < DH_RL2, j
 
 
 @pytest.mark.parametrize("L,V,d", [(9000, 66000, 16), (60, 9000, 520)])
@@ -283,12 +285,14 @@ def test_reference_jumps_over_chunks_and_narrow_tiles(attt, L, V, d):
         assert rel_l2(dh[rows[i]], rdh[i]) < DH_RL2, rows[i]
 
 
-@pytest.mark.parametrize("L,V,d", [(4400, 8000, 64), (8300, 600, 4096)])
+@pytest.mark.parametrize("L,V,d", [(4400, 8000, 64), (8300, 600, 4096), (4400, 8000, 2056)])
 def test_row_tiles_in_groups(attt, L, V, d):
-    """Row tiles whose A exceeds half of L2 (E of the dh contraction in the first
-    shape, h of the logits in the second), so that they are walked in groups of
-    2,048 rows, the last one smaller: sampled rows of every group against the
-    oracle."""
+    """Row tiles whose A exceeds half of L2, so that they are walked in groups of
+    2,048 rows, the last one smaller: E of the dh contraction in the first shape
+    (one column tile, in K pieces) and in the last (nine column tiles, not cut
+    into pieces), h of the logits (three) in the second: sampled rows of every
+    group, all columns, against the oracle.  Groups, pieces and several column
+    tiles together: the test below."""
     h = wk.normal_bf16(L + 5, "h", (L, d), 1.0)
     W = wk.normal_bf16(V + 5, "W", (V, d), 0.02)
     rng = wk.rng_for(L + V + 5, "t")
