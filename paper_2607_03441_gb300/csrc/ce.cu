@@ -56,8 +56,12 @@ struct CeLayout {
 // near kCeEBytes (1 GB), so the workspace stays bounded whatever V is.  Each
 // chunk costs about 20 us of launch, ramp and tail on top of its FLOPs, and E is streamed
 // once from L2 or HBM either way, so wider chunks are faster up to this bound
-// (d 3,584, V 152,064, one chunk against three: L 93 354 against 415 us, L 403
-// 660 against 796, L 2,048 2,350 against 2,390).
+// (d 3,584, V 152,064, calls back to back, one chunk against three: L 93 350
+// against 391 us, L 403 698 against 768, L 2,048 2,640 against 2,670 at the
+// power cap).  They cost memory (workspace at L 2,048 675 against 321 MB) and,
+// where no K pieces shorten it, a longer fp32 accumulation of dh (error against
+// 64 bits at L 2,048, three seeds, 6.21e-4 with three chunks, 6.34e-4 with one;
+// the bf16 rounding of E is nearly all of both).
 static int64_t ce_chunk_max(int64_t L, int64_t V) {
     int64_t vc = kCeEBytes / (2 * L);
     vc = (vc / kCeBN) * kCeBN;

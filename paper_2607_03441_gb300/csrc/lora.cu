@@ -590,10 +590,11 @@ static SkinnyGradPlan skinny_grad_plan(int64_t L, int64_t din, int nproj, const 
     }
     // The grouped form streams every block of both passes over all SMs, but pays
     // for a prep launch and the ends of its tiles: the skinny form wins while its
-    // two passes stream for at most kSkinnyExtra microseconds longer (measured,
-    // grouped against skinny: L 2,048, q and v at r 16, +2.7: 27.0 -> 22.3 us; L
-    // 4,096, 14,336 -> 4,096 at r 32, +4.7: 63 -> 54; L 8,192, 4,096 -> 4,096 and
-    // 1,024 at r 8, +5.4: 58 -> 64; L 6,000, three projections at r 32, +12: 74 -> 85).
+    // two passes stream for at most kSkinnyExtra microseconds longer (device time of
+    // a call in a replayed graph, grouped against skinny: L 2,048, q and v at r 16,
+    // +2.7: 27.9 -> 22.4 us; L 4,096, 14,336 -> 4,096 at r 32, +4.7: 66 -> 54; L
+    // 8,192, 4,096 -> 4,096 and 1,024 at r 8, +5.4: 58 -> 64; L 6,000, three
+    // projections at r 32, +12: 74 -> 85).
     // A rank that is not a multiple of 8 keeps a prep launch (A alone) in both
     // forms; the same line serves it: 40 drawn groups of ranks 4 and 12, mean 31.0
     // us grouped, 25.9 with this line, 26.7 with one 3.5 us lower.

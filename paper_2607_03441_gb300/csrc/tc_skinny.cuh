@@ -13,9 +13,11 @@
 // them; only A of a rank that is not a multiple of 8 (TMA cannot read its rows)
 // is transposed first.
 //
-// Measured on GB300 (call times, grouped form against this one): gradients of
-// q and v of the 7B-class update (2,048 rows, r 16) 27.0 -> 22.3 us, of one
-// projection at 403 rows 19.3 -> 12.5, of four at 411 rows, r 32, 46.5 -> 34.5.
+// Measured on GB300 (device time of a call in a replayed graph, grouped form
+// against this one): gradients of q and v of the 7B-class update (2,048 rows, r
+// 16) 27.9 -> 22.4 us (issued one by one 31.1 -> 24.8), of one 3,584-wide
+// projection at 403 rows 19.6 -> 12.4, of four (3,584, 512, 512, 3,584) at 411
+// rows, r 32, 53.3 -> 19.3.
 // What is left is round trips: setup 0.4 us, first tile 1.3, the K blocks of a
 // CTA at 0.2-0.3 each, barrier 0.8, sum and stores 1.3, barrier 0.9.
 //
