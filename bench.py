@@ -335,7 +335,7 @@ def path_roofline(wl, grad_steps, ms_per_step, peaks, kind):
 
 # The sources the Eq. 10 call is built from (its kernels, the contraction
 # engine they share, the PTX wrappers and the host-side helpers).
-CE_SOURCES = ("ce.cu", "tc_gemm.cuh", "gemm_launch.cuh", "attt_common.cuh", "attt_host.h", "api.cu")
+CE_SOURCES = ("ce.cu", "ce_plan.cuh", "tc_gemm.cuh", "gemm_launch.cuh", "attt_common.cuh", "attt_host.h", "api.cu")
 
 
 def _sources_sha256() -> str:

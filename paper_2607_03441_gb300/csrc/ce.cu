@@ -20,24 +20,15 @@
 // the gradient's factors into alpha and beta, so that the last GEMM2 writes
 //   dh_j = (w_j / L) (acc_j exp(A_j - lse_j) - W_{x_j})
 // directly.  The LM head gets no gradient (frozen; only the adapter trains).
-#include "gemm_launch.cuh"
+#include "ce_plan.cuh"
 
 namespace attt {
 
-constexpr int kCeBN = 256;
-// (max, sum) pairs of sets narrower than those of 256-column tiles, at most: the
-// plan takes narrow tiles only where few tiles would leave SMs idle (L 1 to
-// 20,000, V 256 to 262,144, d 64 to 8,192 on 152 SMs: at most 1,125,316 pairs).
-constexpr int64_t kCeNarrowPairs = 5ll << 18;  // 10 MB
-constexpr int kCeMaxTiles = 1024;  // chunk width at most, in kCeBN columns
-static_assert(kCeMaxTiles * kCeBN <= kCeMaxChunk, "the fp32 range of dh is argued for chunks of kCeMaxChunk columns");
 constexpr int kChunkWarps = 16;  // ce_chunk_kernel: 16 warps of 4 tiles x 8 rows
 constexpr int kChunkRows = 8;    // rows per block: lane & 7
 // fp32 partials of 128 x kCeBN (128 KB each) for the K pieces of the dh
 // contraction (40 MB): two pieces for every SM of a 160-SM part.
 constexpr int kCeSplitRegions = 320;
-// Bound of the chunk's bf16 block E [L, Vc] in bytes.
-constexpr int64_t kCeEBytes = 1024ll << 20;
 
 struct CeLayout {
     int64_t Vc, nblk;
@@ -52,60 +43,13 @@ struct CeLayout {
     size_t bytes;
 };
 
-// Upper bound of the vocab chunk: the chunk's bf16 block E (L x Vc) is kept
-// near kCeEBytes (1 GB), so the workspace stays bounded whatever V is.  Each
-// chunk costs about 20 us of launch, ramp and tail on top of its FLOPs, and E is streamed
-// once from L2 or HBM either way, so wider chunks are faster up to this bound
-// (d 3,584, V 152,064, calls back to back, one chunk against three: L 93 350
-// against 391 us, L 403 698 against 768, L 2,048 2,640 against 2,670 at the
-// power cap).  They cost memory (workspace at L 2,048 675 against 321 MB) and,
-// where no K pieces shorten it, a longer fp32 accumulation of dh (error against
-// 64 bits at L 2,048, three seeds, 6.21e-4 with three chunks, 6.34e-4 with one;
-// the bf16 rounding of E is nearly all of both).
-static int64_t ce_chunk_max(int64_t L, int64_t V) {
-    int64_t vc = kCeEBytes / (2 * L);
-    vc = (vc / kCeBN) * kCeBN;
-    if (vc < 4096) vc = 4096;
-    if (vc > kCeMaxTiles * kCeBN) vc = kCeMaxTiles * kCeBN;
-    const int64_t vmax = round_up(V, kCeBN);
-    if (vc > vmax) vc = vmax;
-    return vc;
-}
-
-// Chunk width and the tiles of both contractions for `sms` SMs.
-struct CePlan {
-    int64_t Vc;
-    TilePlan logits, dh;
-};
-
-// Epilogue sets of a logits tile.
-static int ce_sets(int64_t d) { return cdiv(d, 64) <= kTwoSetBlocks ? 2 : 1; }
-
-// (max, sum) pairs that the sets of a chunk of Vc columns may need.
-static int64_t ce_pairs(int64_t L, int64_t d, int64_t Vc) {
-    const int64_t wide = cdiv(Vc, kCeBN) * ce_sets(d) * L, most = cdiv(Vc, 64) * ce_sets(d) * L;
-    const int64_t narrow = most < kCeNarrowPairs ? most : kCeNarrowPairs;
-    return wide > narrow ? wide : narrow;
-}
-
-static CePlan ce_plan(int64_t L, int64_t d, int64_t V, int regions, int sms) {
-    CePlan p{};
-    const int64_t nchunks = cdiv(V, ce_chunk_max(L, V));
-    p.Vc = round_up(cdiv(V, nchunks), kCeBN);  // equal chunks
-    p.logits = plan_tiles(L, p.Vc, cdiv(d, 64), sms, 0, false, false);
-    const int64_t pairs = ce_pairs(L, d, ce_chunk_max(L, V));
-    while (p.logits.BN < kCeBN && cdiv(p.Vc, p.logits.BN / ce_sets(d)) * L > pairs) p.logits.BN += 64;
-    p.dh = plan_tiles(L, d, cdiv(p.Vc, 64), sms, regions, true, true);
-    return p;
-}
-
 static CeLayout ce_layout(void *ws, int64_t L, int64_t d, int64_t V) {
     CeLayout c{};
     // K pieces of the dh contraction: at most kMaxPieces per tile, of at most
     // two 128-row regions per 256 rows
     const int64_t t2 = 2 * kMaxPieces * cdiv(L, 256) * cdiv(d, kCeBN);
     c.split_regions = (int)(t2 < kCeSplitRegions ? t2 : kCeSplitRegions);
-    c.Vc = ce_chunk_max(L, V);
+    c.Vc = ce_chunk_max(L, d, V);
     c.nblk = cdiv(L, kChunkRows);
     Carve cv{static_cast<char *>(ws), 0};
     c.part = cv.take<float2>((size_t)ce_pairs(L, d, c.Vc));
@@ -380,13 +324,18 @@ size_t attt_ce_workspace_bytes(int64_t L, int64_t d, int64_t V) {
 namespace attt {
 
 // The largest attt_ce_workspace_bytes(L, d, V) over 1 <= L <= Lmax.  The
-// workspace grows with L while the vocabulary chunk Vc stays the same, and Vc
-// (a multiple of kCeBN, clamped to [4096, kCeMaxTiles kCeBN] and to V) only
-// changes where kCeEBytes / (2 L) crosses a multiple of kCeBN, so the maximum is
-// at Lmax or at the last L of one of those ranges.
+// workspace grows with L while the bound of the vocabulary chunk stays the same,
+// and that (ce_chunk_max: a multiple of kCeBN) only changes where kCeEBytes /
+// (2 L) crosses a multiple of kCeBN or the dh tiles pass kCeWholeTiles, so the
+// maximum is at Lmax or at the last L of one of those ranges.
 size_t ce_workspace_bound(int64_t Lmax, int64_t d, int64_t V) {
     if (Lmax < 1) return 0;
     size_t best = attt_ce_workspace_bytes(Lmax, d, V);
+    const int64_t whole = kCeWholeTiles / cdiv(d, 256) * 256;
+    if (whole >= 1 && whole <= Lmax) {
+        const size_t b = attt_ce_workspace_bytes(whole, d, V);
+        if (b > best) best = b;
+    }
     const int64_t budget = kCeEBytes / 2;
     const int64_t vmax = round_up(V, kCeBN) < kCeMaxTiles * kCeBN ? round_up(V, kCeBN) : kCeMaxTiles * kCeBN;
     for (int64_t vc = kCeBN; vc <= vmax; vc += kCeBN) {

@@ -59,7 +59,8 @@ def test_eq10_workspace_holds_little_beside_the_block_and_the_pieces(lib_path, L
     pair per row and column set (128 columns, or 10 MB of narrower ones), row
     terms."""
     from paper_2607_03441_gb300 import attt
-    chunk = min(-(-V // 256) * 256, max(4096, (1 << 30) // (2 * L) // 256 * 256))
+    whole = -(-L // 256) * -(-d // 256) > 64  # chunks of at most 65,536 columns
+    chunk = min(-(-V // 256) * 256, max(4096, (1 << 30) // (2 * L) // 256 * 256), 65536 if whole else 1 << 18)
     got = attt.attt_ce_workspace_bytes(L, d, V)
     regions = min(320, 32 * -(-L // 256) * -(-d // 256))
     pairs = max(chunk // (128 if d <= 1536 else 256) * L, min(5 << 18, chunk // (32 if d <= 1536 else 64) * L))

@@ -1,6 +1,6 @@
-"""The host side of the tile plan and of the tile order, compiled from the
-library's own header: every K piece is stored where the kernel that sums the
-pieces reads it."""
+"""The host side of the tile plans and of the tile order, compiled from the
+library's own headers: every K piece is stored where the kernel that sums the
+pieces reads it, and the plan of Eq. 10 keeps its bounds."""
 import subprocess
 
 import pytest
@@ -10,7 +10,7 @@ from paper_2607_03441_gb300 import build
 PROGRAM = r"""
 #include <cstdio>
 #include <vector>
-#include "gemm_launch.cuh"
+#include "ce_plan.cuh"
 using namespace attt;
 
 // One planned contraction, M x N over K, as launch_planned and launch_gemm cut
@@ -48,11 +48,23 @@ static void walk(int64_t M, int64_t N, int64_t K, int64_t K2, int regions, bool 
     std::printf("%d %d %d %d\n", t.pieces, g.group_m, g.tiles_n, bad);
 }
 
-int main() {
+// The plan of an Eq. 10 call: chunk width and its bound, columns of the longest
+// accumulation of dh, (max, sum) pairs and the pairs there is room for.
+static void eq10(int64_t L, int64_t d, int64_t V, int regions, int sms) {
+    const CePlan p = ce_plan(L, d, V, regions, sms);
+    std::printf("%lld %lld %lld %lld %lld\n", (long long)p.Vc, (long long)ce_chunk_max(L, d, V),
+                (long long)(cdiv(cdiv(p.Vc, 64), p.dh.pieces) * 64),
+                (long long)(cdiv(p.Vc, p.logits.BN / ce_sets(d)) * L), (long long)ce_pairs(L, d, ce_chunk_max(L, d, V)));
+}
+
+int main(int argc, char **) {
     long long M, N, K, K2;
     int regions, tail, b_mn;
-    while (std::scanf("%lld %lld %lld %lld %d %d %d", &M, &N, &K, &K2, &regions, &tail, &b_mn) == 7)
-        walk(M, N, K, K2, regions, tail != 0, b_mn != 0);
+    if (argc > 1)
+        while (std::scanf("%lld %lld %lld %d %d", &M, &N, &K, &regions, &tail) == 5) eq10(M, N, K, regions, tail);
+    else
+        while (std::scanf("%lld %lld %lld %lld %d %d %d", &M, &N, &K, &K2, &regions, &tail, &b_mn) == 7)
+            walk(M, N, K, K2, regions, tail != 0, b_mn != 0);
 }
 """
 
@@ -64,9 +76,9 @@ def walk(tmp_path_factory):
     src.write_text(PROGRAM)
     subprocess.run([build._nvcc(), *build.ARCH, *build.NVCC_FLAGS, str(src), "-o", str(exe)], check=True)
 
-    def run(shapes):
+    def run(shapes, *args):
         text = "\n".join(" ".join(str(int(v)) for v in s) for s in shapes)
-        out = subprocess.run([str(exe)], input=text, capture_output=True, text=True, check=True).stdout
+        out = subprocess.run([str(exe), *args], input=text, capture_output=True, text=True, check=True).stdout
         return [tuple(int(v) for v in line.split()) for line in out.splitlines()]
     return run
 
@@ -109,3 +121,19 @@ def test_pieces_over_a_grid_of_shapes(walk):
     for shape, (_, _, _, bad) in zip(shapes, got):
         assert bad == 0, shape
     assert sum(p > 1 and g > 0 and n > 1 for p, g, n, _ in got) >= 20
+
+
+def test_eq10_chains_and_pairs_stay_within_their_bounds(walk):
+    """Whatever the plan: chunks no wider than the workspace is laid out for,
+    no accumulation of dh over more than 65,536 columns, and no more (max, sum)
+    pairs than there is room for; also on parts with fewer or more SMs."""
+    shapes = [(L, d, V, min(32 * -(-L // 256) * -(-d // 256), 320), sms)
+              for L in (1, 40, 93, 129, 300, 403, 600, 1024, 1500, 2048, 4097, 5888, 8192, 32768)
+              for d in (8, 512, 1032, 1544, 3584, 5120, 8192) for V in (1, 300, 8192, 66000, 152064, 262144, 1000000)
+              for sms in (148, 152, 160, 72)]
+    got = walk(shapes, "eq10")
+    assert len(got) == len(shapes)
+    for shape, (vc, vmax, chain, pairs, room) in zip(shapes, got):
+        assert 0 < vc <= vmax and chain <= 65536 and pairs <= room, shape
+    assert walk([(403, 3584, 152064, 320, 152)], "eq10")[0][0] == 152064  # in pieces: one chunk
+    assert walk([(2048, 3584, 152064, 320, 152)], "eq10")[0][0] == 50688  # whole tiles: three
