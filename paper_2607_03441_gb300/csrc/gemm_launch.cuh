@@ -158,7 +158,7 @@ inline TilePlan plan_tiles(int64_t M, int64_t N, int64_t kb, int sms, int64_t re
 // row and 9.5 column blocks instead of 32 and 2.4.  At 8,192 x 5,120 x
 // 152,064 the logits contractions read 2.6 instead of 5.2 GB from DRAM and the dh
 // contractions 5.8 instead of 9.7 (per chunk, on one GPU; the concurrent tiles
-// drift apart along K, and in four captures the groups read 2.4 to 3.6 and 5.2 to
+// drift apart along K, and in five captures the groups read 2.4 to 3.6 and 5.1 to
 // 8.7), the call at the power cap 15.9 -> 15.0 ms; where A fits (4,096 x 4,096)
 // the logits lose 1% by it.  0: no groups.
 inline int tile_group(int64_t M, int rows_tile, int group, double a_bytes) {
